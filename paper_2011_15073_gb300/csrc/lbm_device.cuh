@@ -8,7 +8,8 @@
 // non-equilibrium moments that carry second velocity moments (e, p_xx, p_xy).
 //
 // The node physics is written once over a value type V:
-//   double -- FP64 arithmetic (IEEE division, square root and pow);
+//   double -- FP64 arithmetic (division, square root and pow as in
+//             lbm_fixed.cuh, about 1 ulp);
 //   float  -- FP32 arithmetic with the approximate special-function unit
 //             (rcp/sqrt/ex2/lg2 .approx, about 1-2 ulp);
 //   F2     -- two nodes in one register pair, the arithmetic on the packed
@@ -21,6 +22,7 @@
 #include <math.h>
 #include <stdint.h>
 
+#include "lbm_fixed.cuh"
 #include "lbm_internal.h"
 #include "lbm_round.cuh"
 
@@ -49,9 +51,9 @@ __device__ __forceinline__ float vfma(float a, float b, float c) { return fmaf(a
 __device__ __forceinline__ F2 vfma(F2 a, F2 b, F2 c) { return F2(__ffma2_rn(a.v, b.v, c.v)); }
 
 // Special functions.
-__device__ __forceinline__ double vrcp(double x) { return 1.0 / x; }
-__device__ __forceinline__ double vsqrt(double x) { return sqrt(x); }
-__device__ __forceinline__ double vpow(double x, double e) { return pow(x, e); }
+__device__ __forceinline__ double vrcp(double x) { return rcp_f64(x); }
+__device__ __forceinline__ double vsqrt(double x) { return sqrt_f64(x); }
+__device__ __forceinline__ double vpow(double x, double e) { return pow_f64(x, e); }
 
 __device__ __forceinline__ float vrcp(float x)
 {
