@@ -66,9 +66,8 @@ aa_even_kernel(typename Store<PREC>::S *__restrict__ A, typename Store<PREC>::Ta
     for (int i = 0; i < 9; i++) f[i] = ldf<PREC>(A, i * P + k, R(rest_f(i)));
 #pragma unroll
     for (int i = 0; i < 5; i++) g[i] = ldf<PREC>(A + 9 * P, i * P + k, R(rest_g(i)));
-    Macro<R> m;
     constexpr int DEV = dev_form<PREC>();
-    const R t = collide<R, FIELD, DEV>(p, f, g, tau_start<TAU, R, FIELD, DEV>(p, f, g, k, [&] { return R(tau[k]); }), m, k);
+    const R t = collide_step<R, FIELD, DEV>(p, f, g, tau_start<TAU, R, FIELD, DEV>(p, f, g, k, [&] { return R(tau[k]); }), k);
     uint32_t rng = rng_init(p.seed, k);
 #pragma unroll
     for (int i = 0; i < 9; i++) stf<PREC>(A, opp(i) * P + k, f[i], R(rest_f(opp(i))), rng);
@@ -86,8 +85,7 @@ __device__ __forceinline__ void odd_node(typename Store<PREC>::S *__restrict__ A
     R f[9], g[5];
     constexpr int DEV = dev_form<PREC>();
     pull<PREC, R, true, DEV>(A, p, x, y, f, g);
-    Macro<R> m;
-    const R t = collide<R, FIELD, DEV>(p, f, g, tau_start<TAU, R, FIELD, DEV>(p, f, g, k, [&] { return R(tau[k]); }), m, k);
+    const R t = collide_step<R, FIELD, DEV>(p, f, g, tau_start<TAU, R, FIELD, DEV>(p, f, g, k, [&] { return R(tau[k]); }), k);
     push<PREC, R>(A, p, x, y, f, g);
     if constexpr (TAU == 0) tau[k] = typename Store<PREC>::TauS(t);
 }

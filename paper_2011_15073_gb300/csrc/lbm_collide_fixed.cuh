@@ -1,0 +1,366 @@
+// lbm_collide_fixed.cuh -- one node's collision of the FP64 storage, mostly in
+// 64-bit fixed point.
+//
+// Why: a warp's FP64 instruction holds a quarter SM's FP64 pipe for 64 cycles
+// on this part (2 lanes per SM and cycle), so the 323 FP64 instructions of
+// the plain collision (96 of them the library's pow()) bound a node update at
+// 2 G nodes/s while nine tenths of the issue slots go unused.  A 64 x 64-bit
+// fixed-point product costs three wide integer multiplies and about four other
+// instructions (some 10 cycles), a sum two instructions, and a conversion to
+// or from FP64 13 to 16.  So the moments, equilibria, forcing, relaxation and
+// the way back run on the integer pipes, and only the porous velocity solve,
+// the square of the strain rate and the reciprocals (39 instructions) stay in
+// FP64, where their range is wide; the power law is evaluated on the logarithm
+// of the shear rate.  Measured, n = 0.8: 1000 x 1100 680 -> 135.6 us per step,
+// 1536^2 1424 -> 274 us (8.6 G nodes/s; the ALU pipe is then 62 % busy, the
+// FP64 pipe 55 %), 64^2 with n = 1 12.1 -> 4.6 us (one warp's latency).
+//
+// Precision: the populations enter exactly (Q60 holds every bit of an FP64
+// value from 2^-7 on, and 2^-60 below), sums are exact, a product is off by at
+// most 2^-60 or so, without bias, and the results are rounded to FP64 once; FP64 arithmetic
+// rounds every one of those operations, to 2^-53 of populations between 0.02
+// and 0.5.  What a node holds outside the ranges below (populations outside
+// (2^-15, 1), |j| >= 1/4, a density outside (1/2, 2), ..., NaN) is left to the
+// plain FP64 collision: collide_fixed() returns false.
+//
+// Q<N> holds a value times 2^N in 64 bits.
+#pragma once
+
+#include "lbm_fixed.cuh"
+
+namespace lbm {
+
+template <int N>
+struct Q {
+    int64_t v;
+};
+template <int N>
+__host__ __device__ __forceinline__ Q<N> operator+(Q<N> a, Q<N> b) { return Q<N>{a.v + b.v}; }
+template <int N>
+__host__ __device__ __forceinline__ Q<N> operator-(Q<N> a, Q<N> b) { return Q<N>{a.v - b.v}; }
+template <int N>
+__host__ __device__ __forceinline__ Q<N> operator*(int k, Q<N> a) { return Q<N>{k * a.v}; }
+// a >> k and a << k: the value halved / doubled k times
+template <int N>
+__host__ __device__ __forceinline__ Q<N> operator>>(Q<N> a, int k) { return Q<N>{a.v >> k}; }
+template <int N>
+__host__ __device__ __forceinline__ Q<N> operator<<(Q<N> a, int k) { return Q<N>{(int64_t)((uint64_t)a.v << k)}; }
+// Another format, rounded to nearest.  (Truncation would do for one step; over
+// many its bias adds up where rounding errors average out.)
+template <int M, int N>
+__host__ __device__ __forceinline__ Q<M> as(Q<N> a)
+{
+    if constexpr (M >= N)
+        return Q<M>{(int64_t)((uint64_t)a.v << (M - N))};
+    else
+        return Q<M>{(a.v + (1ll << (N - M - 1))) >> (N - M)};
+}
+
+// High 64 bits of a signed product, |a|, |b| <= 2^62, to within 3/4, without
+// bias.  Low words are taken as signed and the high words corrected for it,
+// so that all three products are signed ones; the low-low product is dropped.
+__host__ __device__ __forceinline__ int64_t smulhi(int64_t a, int64_t b)
+{
+    const int32_t al = (int32_t)a, bl = (int32_t)b;
+    const int32_t ah = (int32_t)(a >> 32) + (int32_t)((uint32_t)al >> 31);
+    const int32_t bh = (int32_t)(b >> 32) + (int32_t)((uint32_t)bl >> 31);
+    const int64_t s = (int64_t)ah * bl + 0x80000000ll + (int64_t)al * bh;
+    return (int64_t)ah * bh + (s >> 32);
+}
+template <int A, int B>
+__host__ __device__ __forceinline__ Q<A + B - 64> operator*(Q<A> a, Q<B> b) { return Q<A + B - 64>{smulhi(a.v, b.v)}; }
+
+// Whether |a.v| >= 2^K.
+template <int K, int N>
+__host__ __device__ __forceinline__ uint32_t outside(Q<N> a)
+{
+    return (uint32_t)((uint64_t)a.v + (1ull << K) >= (2ull << K));
+}
+
+__host__ __device__ __forceinline__ uint64_t bits_of(double x)
+{
+#ifdef __CUDA_ARCH__
+    return (uint64_t)__double_as_longlong(x);
+#else
+    uint64_t b;
+    memcpy(&b, &x, 8);
+    return b;
+#endif
+}
+__host__ __device__ __forceinline__ double double_of(uint64_t b)
+{
+#ifdef __CUDA_ARCH__
+    return __longlong_as_double((long long)b);
+#else
+    double x;
+    memcpy(&x, &b, 8);
+    return x;
+#endif
+}
+__host__ __device__ __forceinline__ uint32_t hi_word(double x) { return (uint32_t)(bits_of(x) >> 32); }
+
+// x in Q60, exact from 2^-7 on and truncated below 2^-60; 2^-15 <= x < 1.
+__host__ __device__ __forceinline__ Q<60> q60_of_population(double x)
+{
+    const uint64_t b = bits_of(x);
+    const uint64_t m = (b & 0xfffffffffffffull) | (1ull << 52);
+    return Q<60>{(int64_t)((m << 11) >> (1026 - (int)(b >> 52)))};
+}
+// |x| < 2^(62 - N), in Q<N>, to nearest.
+template <int N>
+__host__ __device__ __forceinline__ Q<N> q_of(double x)
+{
+    const uint64_t b = bits_of(x);
+    const uint64_t m = (b & 0xfffffffffffffull) | (1ull << 52);
+    // m 2^(E - 1075) 2^(N + 1) = (m << 11) >> (1085 - N - E), then halved
+    const int right = 1085 - N - ((int)(b >> 52) & 0x7ff);
+    const int64_t q = right > 63 ? 0 : (int64_t)((((m << 11) >> right) + 1) >> 1);
+    const int64_t s = (int64_t)b >> 63;
+    return Q<N>{(q ^ s) - s};
+}
+__host__ __device__ __forceinline__ int clz64(uint64_t x)
+{
+#ifdef __CUDA_ARCH__
+    return __clzll((long long)x);
+#else
+    return x ? __builtin_clzll(x) : 64;
+#endif
+}
+// The nearest FP64 value, ties to even (they are common: a population keeps
+// only a few bits beyond FP64's, and a tie rounded one way would add mass).
+template <int N>
+__host__ __device__ __forceinline__ double double_of(Q<N> a)
+{
+    const int64_t s = a.v >> 63;
+    const uint64_t m = (uint64_t)((a.v ^ s) - s);
+    const int lz = clz64(m);
+    const uint64_t n = m << (lz & 63);   // leading one at bit 63
+    // exponent field 1023 + 63 - lz - N, one less for the leading one
+    const uint32_t l = (uint32_t)n;
+    const uint32_t up = ((l & 0x7ff) + (l >> 11 & 1) + 0x3ff) >> 11;
+    const uint64_t b = ((uint64_t)(1023 + 62 - N - lz) << 52) + (n >> 11) + up;
+    return double_of(m == 0 ? 0ull : b | ((uint64_t)s & (1ull << 63)));
+}
+
+// The per-case constants in fixed point, built on the host from the same
+// values as the FP64 ones; ok: every one within the range its format holds.
+struct FixedParams {
+    int ok;
+    Q<64> buoy;          // eps g beta, below 1/4
+    Q<61> omegaT, s_p;   // below 2
+    Q<62> s_e3;          // s_e / 3
+    Q<60> inv_eps;       // below 4
+    Q<62> nm1;           // n - 1, below 1 in size
+    Q<57> log_scale;     // log2(3/2 gamma_scale), in [0, 32)
+    Q<57> log_g1, log_g2;
+};
+
+template <int N>
+inline Q<N> q_host(double x, int &ok)
+{
+    if (!(fabs(x) < ldexp(1.0, 62 - N))) {
+        ok = 0;
+        return Q<N>{0};
+    }
+    return Q<N>{llrintl(ldexpl((long double)x, N))};
+}
+inline FixedParams fixed_params(double eps, double gbeta, double omegaT, double s_e, double s_p, double n,
+                                double gamma_scale, double gamma1, double gamma2, int clamp_mode)
+{
+    FixedParams f;
+    f.ok = clamp_mode == 1 || n == 1.0;   // the literal law jumps at both ends unless n = 1
+    f.buoy = q_host<64>(eps * gbeta, f.ok);
+    f.omegaT = q_host<61>(omegaT, f.ok);
+    f.s_p = q_host<61>(s_p, f.ok);
+    f.s_e3 = q_host<62>(s_e / 3.0, f.ok);
+    f.inv_eps = q_host<60>(1.0 / eps, f.ok);
+    f.nm1 = q_host<62>(n - 1.0, f.ok);
+    auto log2_of = [&](double x, double least) {
+        const long double l = log2l((long double)x);
+        if (!(l >= least && l < 32.0L)) {
+            f.ok = 0;
+            return Q<57>{0};
+        }
+        return Q<57>{llrintl(ldexpl(l, 57))};
+    };
+    f.log_scale = log2_of(1.5 * gamma_scale, 0.0);
+    f.log_g1 = log2_of(gamma1, -32.0);
+    f.log_g2 = log2_of(gamma2, -32.0);
+    return f;
+}
+
+__host__ __device__ __forceinline__ double rcp_or_ieee(double x)
+{
+#ifdef __CUDA_ARCH__
+    return rcp_f64(x);
+#else
+    return 1.0 / x;
+#endif
+}
+__host__ __device__ __forceinline__ double sqrt_or_ieee(double x)
+{
+#ifdef __CUDA_ARCH__
+    return sqrt_f64(x);
+#else
+    return sqrt(x);
+#endif
+}
+
+// 1 / r in Q61 for a density r in Q60, 1/2 < r < 2: a 23-bit approximation
+// x, then x (1 + e + e^2) with e = 1 - r x, |e| < 2^-21.
+__host__ __device__ __forceinline__ Q<61> rcp_density(Q<60> r)
+{
+#ifdef __CUDA_ARCH__
+    float y;
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(__uint2float_rn((uint32_t)(r.v >> 30))));   // 2^-30 / r
+    const uint32_t x = __float2uint_rn(y * 0x1p60f);                                             // 2^30 / r
+#else
+    const uint32_t x = (uint32_t)lrintf(1.0f / (float)(uint32_t)(r.v >> 30) * 0x1p60f);
+#endif
+    const uint32_t rh = (uint32_t)(r.v >> 32), rl = (uint32_t)r.v;
+    // r x in Q58 (Q60 Q30 2^-32), below 2^60
+    const int64_t e = (1ll << 58) - (int64_t)((uint64_t)rh * x + ((uint64_t)rl * x >> 32));
+    const int32_t es = (int32_t)(e >> 10);                                // Q48
+    const int64_t c = e + (int64_t)((uint64_t)((int64_t)es * es) >> 38);  // e + e^2 in Q58
+    // x c: Q30 Q58, to Q61; c is below 2^38 in size
+    const int64_t ch = c >> 20;
+    const uint32_t cl = (uint32_t)c & 0xfffffu;
+    return Q<61>{((int64_t)x << 31) + (((int64_t)x * ch + (int64_t)(((uint64_t)x * cl) >> 20)) >> 7)};
+}
+
+// The collision of a node in place (full values f_i, g_i; the formulas of
+// collide() in lbm_device.cuh): f, g become the post-collision populations and
+// tau the new relaxation time (tau_prev the one the collision starts from).
+// heK, eK, c1, eFsK: the node's porous coefficients.  Returns false, with
+// nothing changed, where a value leaves the ranges of its format.
+__host__ __device__ __forceinline__ bool collide_fixed(const FixedParams &p, double nu3, bool quadratic_drag, double heK, double eK, double c1,
+                                                       double eFsK, double f[9], double g[5], double &tau)
+{
+    // ranges of the inputs: populations in [2^-15, 1), |g| < 1, tau in [1/4, 2^10)
+    uint32_t bad = 0;
+    for (int i = 0; i < 9; i++) bad |= (uint32_t)(hi_word(f[i]) - 0x3f000000u >= 0x00f00000u);
+    for (int i = 0; i < 5; i++) bad |= (uint32_t)((hi_word(g[i]) & 0x7fffffffu) >= 0x3ff00000u);
+    bad |= (uint32_t)(hi_word(tau) - 0x3fd00000u >= 0x00c00000u);
+    if (bad) return false;
+
+    Q<60> F[9], G[5];
+    for (int i = 0; i < 9; i++) F[i] = q60_of_population(f[i]);
+    for (int i = 0; i < 5; i++) G[i] = q_of<60>(g[i]);
+    constexpr Q<60> one{1ll << 60};
+    // moments; r0 = rho - 1, e and ep without their rest values -2 and 1
+    const Q<60> p13 = F[1] + F[3], p24 = F[2] + F[4], p57 = F[5] + F[7], p68 = F[6] + F[8];
+    const Q<60> d13 = F[1] - F[3], d24 = F[2] - F[4], d57 = F[5] - F[7], d68 = F[6] - F[8];
+    const Q<60> sax = p13 + p24, sdg = p57 + p68;
+    const Q<60> rho = F[0] + sax + sdg, r0 = rho - one;
+    const Q<60> dx = d57 - d68, dy = d57 + d68;
+    const Q<60> jx = d13 + dx, jy = d24 + dy;
+    const Q<60> e = (sdg << 1) - (F[0] << 2) - sax + (one << 1);
+    const Q<60> ep = (F[0] << 2) - (sax << 1) + sdg - one;
+    const Q<60> qx = dx - (d13 << 1), qy = dy - (d24 << 1);
+    const Q<60> pxx = p13 - p24, pxy = p57 - p68;
+    const Q<60> g13 = G[1] + G[3], g24 = G[2] + G[4], s14 = g13 + g24;
+    const Q<60> t0 = G[0] + s14 - (one >> 1);   // T - T_m
+    const Q<60> n1 = G[1] - G[3], n2 = G[2] - G[4], n4 = g13 - g24;
+    const Q<60> n3 = s14 - (G[0] << 2) + Q<60>{384307168202282325}, n3n = 3 * n3 + (t0 << 1);   // without its rest value -1/3
+    // density in (1/2, 2), |j| < 1/4, |T - T_m| < 1, ...
+    bad |= (uint32_t)((uint64_t)rho.v - (1ull << 59) >= (3ull << 59));
+    bad |= outside<58>(jx) | outside<58>(jy) | outside<60>(t0) | outside<59>(n1) | outside<59>(n2) | outside<59>(n4) |
+           outside<60>(n3n);
+    if (bad) return false;
+
+    // velocity v and the porous solve u = v / (c0 + sqrt(c0^2 + c1 |v|)), the latter in FP64
+    const Q<61> irho = rcp_density(rho);
+    const Q<62> buoy = as<62>(t0) * p.buoy;   // eps g beta (T - T_m)
+    const Q<62> vx = as<62>(as<64>(jx) * irho), vy = as<62>(as<64>(jy) * irho) + (buoy >> 1);
+    if (outside<60>(vx) | outside<60>(vy)) return false;
+    const double nu_prev = fma(tau, 1.0 / 3.0, -1.0 / 6.0);
+    const double c0 = fma(heK, nu_prev, 0.5);
+    double iden, drag = -eK * nu_prev;
+    if (quadratic_drag) {
+        const Q<64> wx = as<64>(vx), wy = as<64>(vy);
+        const double vmag = sqrt_or_ieee(double_of(wx * wx + wy * wy));
+        iden = rcp_or_ieee(c0 + sqrt_or_ieee(fma(c0, c0, c1 * vmag)));
+        drag = fma(-eFsK, vmag * iden, drag);
+    } else {
+        iden = rcp_or_ieee(c0 + c0);
+    }
+    // 1 / den in (0, 1], |drag| < 1, coefficients for which 2^-64 in |v|^2 is below FP64's own rounding
+    bad |= (uint32_t)(hi_word(iden) > 0x3ff00000u) | (uint32_t)((hi_word(drag) & 0x7fffffffu) >= 0x3ff00000u);
+    bad |= (uint32_t)(hi_word(c1) >= 0x40100000u) | (uint32_t)(hi_word(eFsK) >= 0x40200000u);
+    if (bad) return false;
+    const Q<62> idq = q_of<62>(iden);
+    const Q<62> drq = q_of<62>(drag);
+    const Q<64> ux = as<64>(as<64>(vx) * idq), uy = as<64>(as<64>(vy) * idq);
+    const Q<62> fx = drq * ux, fy = drq * uy + buoy;
+    // equilibria: rho u u / eps
+    const Q<60> rie = as<60>(as<61>(rho) * p.inv_eps);
+    const Q<64> xx = ux * ux, yy = uy * uy, xy = ux * uy;
+    const Q<60> Kxx = (xx - yy) * rie, Kxy = xy * rie, K3 = 3 * ((xx + yy) * rie);
+    const Q<60> e_eq = K3 - (r0 << 1), ep_eq = r0 - K3;
+    const Q<60> en = e - e_eq, pn = pxx - Kxx, cn = pxy - Kxy;
+    if (outside<60>(fx) | outside<60>(fy) | outside<57>(pn) | outside<57>(cn)) return false;
+    const Q<64> Fx = as<64>(fx), Fy = as<64>(fy);
+    double D = 1.0;
+    if (p.nm1.v != 0) {
+        // shear rate: gamma = 3 / (2 rho tau) sqrt(4 (1.4 tau en / 6)^2 + pn^2 + 4 cn^2), the square in FP64
+        const double a = double_of(en) * tau, b = double_of(pn), c = double_of(cn << 1);
+        const double ss = fma(a * (4.0 * (1.4 / 6.0) * (1.4 / 6.0)), a, fma(b, b, c * c));
+        if (hi_word(ss) >= 0x40500000u) return false;   // below 64
+        const double r = rcp_or_ieee(double_of(rho) * tau);
+        // log2 of the non-dimensional rate; a square below 2^-100 counts as 2^-100, far below gamma_1
+        const uint64_t sb = bits_of(ss * (r * r)), low = (uint64_t)(1023 - 100) << 52;
+        Q<57> L = p.log_scale + Q<57>{log2_sqrt_q57(sb < low ? low : sb)};
+        if (L.v < p.log_g1.v) L = p.log_g1;
+        if (L.v > p.log_g2.v) L = p.log_g2;
+        D = exp2_q56(as<56>(L * p.nm1).v);
+    }
+    const double tau_new = fma(nu3, D, 0.5);
+    const double w = rcp_or_ieee(tau_new);
+    if (hi_word(w) >= 0x40000000u) return false;   // tau > 1/2
+    const Q<61> wq = q_of<61>(w);
+    // forcing moments
+    const Q<64> xX = ux * Fx, yY = uy * Fy;
+    const Q<60> R = (xX + yY) * rie;   // rho u.F / eps
+    const Q<60> Fxx = ((xX - yY) * rie) << 1, Fxy = (ux * Fy + uy * Fx) * rie;
+    // post-collision moments over their squared norms
+    const Q<64> n9{2049638230412172402}, n180{102481911520608620}, n6{3074457345618258603}, n60{307445734561825860};
+    const Q<60> rux = as<60>(as<61>(rho) * ux), ruy = as<60>(as<61>(rho) * uy);
+    const Q<60> rFx = as<60>(as<61>(rho) * Fx), rFy = as<60>(as<61>(rho) * Fy);
+    const Q<60> a0 = r0 * n9;
+    const Q<60> a1 = (7 * e_eq - (e << 1) + 9 * R) * n180;
+    const Q<60> a2 = (7 * ep_eq - (ep << 1) - 9 * R) * n180;
+    const Q<60> a3 = (rux + (rFx >> 1)) * n6, a5 = (ruy + (rFy >> 1)) * n6;
+    const Q<60> a4 = Q<60>{0} - (qx + 6 * rux + (rFx << 1)) * n60, a6 = Q<60>{0} - (qy + 6 * ruy + (rFy << 1)) * n60;
+    const Q<60> a7 = (pxx + Fxx - as<60>(as<64>(pn + (Fxx >> 1)) * wq)) >> 2;
+    const Q<60> a8 = (pxy + Fxy - as<60>(as<64>(cn + (Fxy >> 1)) * wq)) >> 2;
+    const Q<60> ax = a0 - a1 - (a2 << 1) + Q<60>{128102389400760775}, dg = a0 + (a1 << 1) + a2 + Q<60>{32025597350190194};
+    const Q<60> xa = a3 - (a4 << 1), ya = a5 - (a6 << 1), xd = a3 + a4, yd = a5 + a6;
+    const Q<60> f0 = a0 + ((a2 - a1) << 2) + Q<60>{512409557603043100};
+    // thermal moments
+    const Q<61> T = as<61>(t0 + (one >> 1));
+    const Q<60> n1n = n1 - as<60>(T * ux), n2n = n2 - as<60>(T * uy);
+    const Q<60> n1s = n1 - as<60>(as<62>(n1n) * p.omegaT), n2s = n2 - as<60>(as<62>(n2n) * p.omegaT);
+    const Q<60> n3s = n3 - as<62>(n3n) * p.s_e3, n4s = n4 - as<60>(as<63>(n4) * p.s_p);
+    const Q<64> n5{3689348814741910323}, n20{922337203685477581};
+    const Q<60> t5 = t0 * n5, t20 = t5 + n3s * n20 + Q<60>{96076792050570581}, q4 = n4s >> 2;
+    const Q<60> gx = t20 + q4, gy = t20 - q4, h1 = n1s >> 1, h2 = n2s >> 1;
+    tau = tau_new;
+    f[0] = double_of(f0);
+    const Q<60> axp = ax + a7, axm = ax - a7, sxy = xd + yd, dxy = xd - yd, dgp = dg + a8, dgm = dg - a8;
+    f[1] = double_of(axp + xa);
+    f[2] = double_of(axm + ya);
+    f[3] = double_of(axp - xa);
+    f[4] = double_of(axm - ya);
+    f[5] = double_of(dgp + sxy);
+    f[6] = double_of(dgm - dxy);
+    f[7] = double_of(dgp - sxy);
+    f[8] = double_of(dgm + dxy);
+    g[0] = double_of(t5 - n3s * n5 + Q<60>{192153584101141163});
+    g[1] = double_of(gx + h1);
+    g[2] = double_of(gy + h2);
+    g[3] = double_of(gx - h1);
+    g[4] = double_of(gy - h2);
+    return true;
+}
+
+}  // namespace lbm

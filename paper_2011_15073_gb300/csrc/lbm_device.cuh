@@ -8,8 +8,9 @@
 // non-equilibrium moments that carry second velocity moments (e, p_xx, p_xy).
 //
 // The node physics is written once over a value type V:
-//   double -- FP64 arithmetic (division, square root and pow as in
-//             lbm_fixed.cuh, about 1 ulp);
+//   double -- FP64 arithmetic (IEEE division, square root and pow); a time
+//             step's collision runs in 64-bit fixed point where it may
+//             (lbm_collide_fixed.cuh, collide_step below);
 //   float  -- FP32 arithmetic with the approximate special-function unit
 //             (rcp/sqrt/ex2/lg2 .approx, about 1-2 ulp);
 //   F2     -- two nodes in one register pair, the arithmetic on the packed
@@ -22,6 +23,9 @@
 #include <math.h>
 #include <stdint.h>
 
+#include <type_traits>
+
+#include "lbm_collide_fixed.cuh"
 #include "lbm_fixed.cuh"
 #include "lbm_internal.h"
 #include "lbm_round.cuh"
@@ -51,9 +55,9 @@ __device__ __forceinline__ float vfma(float a, float b, float c) { return fmaf(a
 __device__ __forceinline__ F2 vfma(F2 a, F2 b, F2 c) { return F2(__ffma2_rn(a.v, b.v, c.v)); }
 
 // Special functions.
-__device__ __forceinline__ double vrcp(double x) { return rcp_f64(x); }
-__device__ __forceinline__ double vsqrt(double x) { return sqrt_f64(x); }
-__device__ __forceinline__ double vpow(double x, double e) { return pow_f64(x, e); }
+__device__ __forceinline__ double vrcp(double x) { return 1.0 / x; }
+__device__ __forceinline__ double vsqrt(double x) { return sqrt(x); }
+__device__ __forceinline__ double vpow(double x, double e) { return pow(x, e); }
 
 __device__ __forceinline__ float vrcp(float x)
 {
@@ -78,10 +82,18 @@ __device__ __forceinline__ float vpow(float x, float e) { return vexp2(e * __log
 __device__ __forceinline__ F2 vrcp(F2 a) { return F2(vrcp(a.v.x), vrcp(a.v.y)); }
 __device__ __forceinline__ F2 vsqrt(F2 a) { return F2(vsqrt(a.v.x), vsqrt(a.v.y)); }
 
+// Constants only the FP64 kernels have: those of the fixed-point collision.
+template <class V>
+struct PhysFixed {};
+template <>
+struct PhysFixed<double> {
+    FixedParams fixed;
+};
+
 // Per-case constants in the compute type V (built on the host from
 // lbm_lattice by make_params below).
 template <class V>
-struct Phys {
+struct Phys : PhysFixed<V> {
     int nx, ny;
     int64_t pitch;   // elements between rows of a plane
     int64_t plane;   // elements between planes
@@ -163,6 +175,9 @@ inline Phys<V> make_params(const lbm_ctx *c)
     p.tau0 = V(L.tau0);
     p.nu3 = V(3.0 * L.nu_ref);
     p.seed = step_seed((uint64_t)c->steps, run_word(c->opts.seed));
+    if constexpr (std::is_same<V, double>::value)
+        p.fixed = fixed_params(L.eps, L.gbeta, 1.0 / L.tauT, L.s_e, L.s_p, L.n, L.gamma_scale, L.gamma1, L.gamma2,
+                               L.clamp_mode);
     return p;
 }
 
@@ -813,6 +828,26 @@ __device__ __forceinline__ V collide(const Phys<V> &p, V f[9], V g[5], V tau_pre
     g[3] = t03 - h1 + t4;
     g[4] = t03 - h2 - t4;
     return tau;
+}
+
+// The collision of a time step: collide() without the macroscopic values, and
+// for FP64 storage in fixed point wherever the node's values are in its ranges
+// and the case admits it (FixedParams::ok: parameters in range, and a law of
+// the viscosity that is continuous -- at a jump of the literal law the last
+// bits decide which side a node is on, so its runs keep the FP64 arithmetic).
+template <class V, int FIELD = 2, int DEV = 0>
+__device__ __forceinline__ V collide_step(const Phys<V> &p, V f[9], V g[5], V tau_prev, int64_t k)
+{
+    if constexpr (std::is_same<V, double>::value && DEV == 0) {
+        if (p.fixed.ok) {
+            const Porous<V> q = porous_at<V, FIELD>(p, k);
+            V tau = tau_prev;
+            if (collide_fixed(p.fixed, p.nu3, p.eFe > 0.0, q.heK, q.eK, q.c1, q.eFsK, f, g, tau))
+                return tau;
+        }
+    }
+    Macro<V> m;
+    return collide<V, FIELD, DEV>(p, f, g, tau_prev, m, k);
 }
 
 }  // namespace lbm

@@ -1,24 +1,25 @@
-// lbm_fixed.cuh -- FP64 special functions for a GPU whose FP64 pipe is slow.
+// lbm_fixed.cuh -- 64-bit fixed-point logarithm and exponential, and FP64
+// reciprocal and square root, for a GPU whose FP64 pipe is slow.
 //
 // On this part one FP64 instruction of a warp holds a quarter SM's FP64 pipe
 // for 64 cycles, however many of its lanes are active (measured), while the
-// integer pipe issues a warp instruction every cycle or two.  A library pow()
-// costs 96 FP64 instructions (measured), a third of a node update.  The power
-// here runs in 64-bit fixed point on the integer pipe instead, without FP64
-// instructions, and the reciprocal (3 FP64 instructions) and the square root
-// (6) start from the special-function unit's approximation.
+// integer pipes take a warp instruction every cycle or two.  The library's
+// pow() costs 96 FP64 instructions, an IEEE division 5 and a square root 9
+// (measured).  Here the logarithm and the exponential run in fixed point,
+// without FP64 instructions, and the reciprocal (3) and the square root (5)
+// start from the special-function unit's approximation.
 //
-// Method of the power (table-driven logarithm and exponential as in Tang,
-// "Table-driven implementation of the logarithm function in IEEE
-// floating-point arithmetic", ACM TOMS 16, 1990, carried out in fixed point):
+// Method (table-driven as in Tang, "Table-driven implementation of the
+// logarithm function in IEEE floating-point arithmetic", ACM TOMS 16, 1990,
+// carried out in fixed point):
 //   x = 2^E m, 1 <= m < 2; an 11-bit c from the top seven bits of m
 //   makes m c = 1 + z with 0 <= z < 2^-6.8, and the product is exact in 64 bits;
 //   log2 x = E - log2 c + log2(1 + z), the last by its Taylor series;
 //   2^y = 2^floor(y) 2^(j/64) 2^r with 0 <= r < 1/64, the last by its Taylor
 //   series.
-// Qn below means an integer holding the value times 2^n.  Error of the result
-// against 80- and 128-bit arithmetic: under 0.6 units in the last place for
-// |e| <= 1 (0.7 for |e| < 2).
+// Qn below means an integer holding the value times 2^n.  The logarithm is
+// within 2^-56, the exponential within 0.53 units in the last place (against
+// 80-bit arithmetic).
 #pragma once
 
 #include <math.h>
@@ -105,10 +106,9 @@ static const LogEntry kLog2Table[128] = {LBM_LOG_TABLE};
 static const unsigned long long kExp2Table[64] = {LBM_EXP_TABLE};
 #endif
 
-// log2 of the mantissa and exponent of x (normal, positive) in Q57.
-__host__ __device__ __forceinline__ int64_t log2_q57(uint64_t bits)
+// log2 of the mantissa of x (normal, positive) in Q57.
+__host__ __device__ __forceinline__ int64_t log2_mantissa_q57(uint64_t bits)
 {
-    const int E = (int)(bits >> 52) - 1023;
     const LogEntry t = kLog2Table[(bits >> 45) & 127];
     const uint64_t m = (bits & 0xfffffffffffffull) | (1ull << 52);
     // z in Q63 exactly; z' = 32 z in Q64 (below 0.28)
@@ -122,7 +122,12 @@ __host__ __device__ __forceinline__ int64_t log2_q57(uint64_t bits)
     uint64_t u = 0x0000f6384ee1d020ull - mulhi(z, (uint64_t)v << 11);
     u = 0x002e2a8eca5705fcull - mulhi(z, u);
     u = 0x0b8aa3b295c17f0cull - mulhi(z, u);
-    return ((int64_t)E << 57) + (int64_t)t.t + (int64_t)(mulhi(z, u) >> 7);
+    return (int64_t)t.t + (int64_t)(mulhi(z, u) >> 7);
+}
+// log2 sqrt(x) in Q57, 2^-126 <= x < 2^126.
+__host__ __device__ __forceinline__ int64_t log2_sqrt_q57(uint64_t bits)
+{
+    return ((int64_t)((int)(bits >> 52) - 1023) << 56) + (log2_mantissa_q57(bits) >> 1);
 }
 
 // 2^(p / 2^56) as a double.
@@ -146,25 +151,6 @@ __host__ __device__ __forceinline__ double exp2_q56(int64_t p)
     double d;
     memcpy(&d, &bits, 8);
     return d;
-}
-
-// Whether pow_fixed() takes x and e: x positive and normal with
-// 2^-60 <= x < 2^60, |e| < 2 (so the result is normal).
-__host__ __device__ __forceinline__ bool pow_in_range(uint64_t xb, uint64_t eb)
-{
-    return (uint32_t)(xb >> 52) - (1023u - 60u) < 120u && ((uint32_t)(eb >> 52) & 0x7ff) < 1024u;
-}
-
-// x^e for arguments that pow_in_range() admits.
-__host__ __device__ __forceinline__ double pow_fixed(uint64_t xb, uint64_t eb)
-{
-    const int64_t L = log2_q57(xb);
-    // |e| = 2^(E - 1023) m / 2^52; |L| m in Q56, then |e L| in Q56
-    const uint64_t m = (eb & 0xfffffffffffffull) | (1ull << 52);
-    const int right = 1023 - ((int)(eb >> 52) & 0x7ff);
-    const uint64_t q = mulhi(L < 0 ? (uint64_t)-L : (uint64_t)L, m << 11) + 1;   // 1: the mean of what mulhi() drops
-    const int64_t p = right > 62 ? 0 : (int64_t)(((q << 1 >> right) + 1) >> 1);
-    return exp2_q56((L < 0) != ((int64_t)eb < 0) ? -p : p);
 }
 
 #ifdef __CUDACC__
@@ -191,14 +177,6 @@ __device__ __forceinline__ double sqrt_f64(double x)
     const double s1 = fma(fma(-s, s, x), h, s);
     const double r = fma(fma(-s1, s1, x), h, s1);
     return __double2hiint(x) < 0x00100000 && __double2hiint(x) >= 0 ? 0.0 : r;
-}
-
-// x^e; the library's pow() where the fixed-point one does not apply.
-static __device__ __noinline__ double pow_library(double x, double e) { return pow(x, e); }
-__device__ __forceinline__ double pow_f64(double x, double e)
-{
-    const uint64_t xb = (uint64_t)__double_as_longlong(x), eb = (uint64_t)__double_as_longlong(e);
-    return pow_in_range(xb, eb) ? pow_fixed(xb, eb) : pow_library(x, e);
 }
 #endif
 

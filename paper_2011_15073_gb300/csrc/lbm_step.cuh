@@ -29,9 +29,8 @@ __device__ __forceinline__ void step_node(const typename Store<PREC>::S *__restr
     R f[9], g[5];
     constexpr int DEV = dev_form<PREC>();
     pull<PREC, R, false, DEV>(src, p, x, y, f, g);
-    Macro<R> m;
     const R t0 = tau_start<TAU, R, FIELD, DEV>(p, f, g, k, [&] { return R(tsrc[k]); });
-    const R tau = collide<R, FIELD, DEV>(p, f, g, t0, m, k);
+    const R tau = collide_step<R, FIELD, DEV>(p, f, g, t0, k);
     uint32_t rng = rng_init(seed, k);   // random bits of the stochastic-rounding storages
 #pragma unroll
     for (int i = 0; i < 9; i++) stf<PREC>(dst, i * p.plane + k, f[i], R(rest_f(i)), rng);
