@@ -339,13 +339,24 @@ static cudaError_t init_t(lbm_ctx *c)
     return cudaGetLastError();
 }
 
+// Threads per block of the one-node-per-thread FP64 step: single warps, so
+// that a row that is not a multiple of a larger block leaves no idle warps and
+// the scheduler spreads the rest evenly over the SMs' four partitions, each of
+// which has its own FP64 pipe (160^2: 128 threads 9.1 us in fixed point and
+// 36.1 us in FP64 arithmetic, 64 threads 7.1 and 24.7, 32 threads 6.8 and
+// 19.2; 1000 x 1100: the same for all).  A grid with no more warps than the
+// 608 partitions of the chip has nothing to spread, and starts faster in
+// blocks of two (64^2: 4.6 against 4.9 us).
+static int f64_block(const lbm_ctx *c) { return (int64_t)((c->nx + 31) / 32) * c->ny <= 608 ? 64 : 32; }
+
 template <int PREC, int TAU>
 static cudaError_t step_buffers_tau(lbm_ctx *c, const void *src, void *dst, const void *tsrc, void *tdst)
 {
     using St = Store<PREC>;
     if constexpr (PREC == LBM_F64) {
         auto *kern = c->d_da ? step_kernel<PREC, 1, TAU> : step_kernel<PREC, 0, TAU>;
-        kern<<<node_grid(c, 128), 128, 0, c->stream>>>(
+        const int bx = f64_block(c);
+        kern<<<node_grid(c, bx), bx, 0, c->stream>>>(
             (const typename St::S *)src, (typename St::S *)dst, (const typename St::TauS *)tsrc,
             (typename St::TauS *)tdst, make_params<typename St::R>(c));
     } else {
