@@ -64,7 +64,14 @@ int capture_steps(lbm_ctx *c, int G, int par)
     }
     cudaError_t e = cudaSuccess;
     const bool sr = lbm::rounds_stochastically(c->opts.prec);
-    for (int i = 0; i < G && e == cudaSuccess; i++) {
+    int i = 0;
+    // an even number of double steps, so that they too end in the buffer they began in
+    if (lbm::two_steps(c))
+        for (; i + 4 <= G && e == cudaSuccess; i += 4) {
+            e = lbm::launch_two_steps(c);
+            if (e == cudaSuccess) e = lbm::launch_two_steps(c);
+        }
+    for (; i < G && e == cudaSuccess; i++) {
         c->capture_s = sr ? i : -1;   // seeds from d_step_base + i (lbm_kernels.cu)
         e = lbm::launch_step(c);
     }
@@ -482,6 +489,11 @@ int lbm_step(lbm_ctx *c, int64_t k)
             t += G;
         }
     }
+    if (lbm::two_steps(c))
+        for (; t + 2 <= k; t += 2) {
+            CK(lbm::launch_two_steps(c));
+            c->steps += 2;
+        }
     for (; t < k; t++) {
         CK(lbm::launch_step(c));
         c->steps++;   // also the stochastic rounding's step counter

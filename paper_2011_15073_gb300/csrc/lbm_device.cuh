@@ -54,6 +54,35 @@ __device__ __forceinline__ double vfma(double a, double b, double c) { return fm
 __device__ __forceinline__ float vfma(float a, float b, float c) { return fmaf(a, b, c); }
 __device__ __forceinline__ F2 vfma(F2 a, F2 b, F2 c) { return F2(__ffma2_rn(a.v, b.v, c.v)); }
 
+// Rounding of the few sums of a product that are not written as vfma().  The
+// nodes a kernel updates one at a time in FP32 (those of the wall tiles) fuse
+// them, the packed ones round the product first, and a node's rounding must not
+// depend on the kernel that updates it: FP32 runs are compared bit for bit
+// between kernels.  So a packed kernel that takes wall nodes too says which
+// components of its pair are to be rounded as single nodes (SingleLanes).
+struct AsUsual {};
+struct SingleLanes {
+    bool x, y;
+};
+// c - a b
+__device__ __forceinline__ double nmad(double a, double b, double c, AsUsual) { return c - a * b; }
+__device__ __forceinline__ float nmad(float a, float b, float c, AsUsual) { return fmaf(-a, b, c); }
+__device__ __forceinline__ F2 nmad(F2 a, F2 b, F2 c, AsUsual) { return c - a * b; }
+__device__ __forceinline__ F2 nmad(F2 a, F2 b, F2 c, SingleLanes z)
+{
+    const F2 two = c - a * b, one = vfma(-a, b, c);
+    return F2(z.x ? one.v.x : two.v.x, z.y ? one.v.y : two.v.y);
+}
+// c + a b
+__device__ __forceinline__ double pmad(double a, double b, double c, AsUsual) { return c + a * b; }
+__device__ __forceinline__ float pmad(float a, float b, float c, AsUsual) { return fmaf(a, b, c); }
+__device__ __forceinline__ F2 pmad(F2 a, F2 b, F2 c, AsUsual) { return c + a * b; }
+__device__ __forceinline__ F2 pmad(F2 a, F2 b, F2 c, SingleLanes z)
+{
+    const F2 two = c + a * b, one = vfma(a, b, c);
+    return F2(z.x ? one.v.x : two.v.x, z.y ? one.v.y : two.v.y);
+}
+
 // Special functions.
 __device__ __forceinline__ double vrcp(double x) { return 1.0 / x; }
 __device__ __forceinline__ double vsqrt(double x) { return sqrt(x); }
@@ -239,9 +268,11 @@ struct Store<LBM_F32> {
     static __device__ __forceinline__ void st(S *p, int64_t k, R v, R, uint32_t = 0) { p[k] = v; }
     static __device__ __forceinline__ R ldd(const S *p, int64_t k, R rest) { return p[k] - rest; }
     static __device__ __forceinline__ void sdv(S *p, int64_t k, R d, R rest, uint32_t &) { p[k] = d + rest; }
+    using Raw = float2;   // a stored pair as it is loaded
+    static __device__ __forceinline__ F2 of_raw(Raw r, float rest) { return F2(r) - F2(rest); }
     static __device__ __forceinline__ F2 ldd2(const S *p, int64_t k, float rest)
     {
-        return F2(*reinterpret_cast<const float2 *>(p + k)) - F2(rest);
+        return of_raw(*reinterpret_cast<const float2 *>(p + k), rest);
     }
     static __device__ __forceinline__ void sdv2(S *p, int64_t k, F2 d, float rest, uint32_t &)
     {
@@ -261,6 +292,8 @@ struct Store<LBM_F32D> {
     using S = float;
     using R = float;
     using TauS = float;
+    using Raw = float2;
+    static __device__ __forceinline__ F2 of_raw(Raw r, float) { return F2(r); }
     static __device__ __forceinline__ R ld(const S *p, int64_t k, R rest) { return rest + p[k]; }
     static __device__ __forceinline__ void st(S *p, int64_t k, R v, R rest, uint32_t = 0) { p[k] = v - rest; }
     static __device__ __forceinline__ F2 ld2(const S *p, int64_t k, float rest)
@@ -568,9 +601,18 @@ struct Porous {
 };
 // FIELD: 0 the uniform permeability, 1 the per-node field, 2 decide at run
 // time from p.da (kernels that know which one they run pass 0 or 1, so the
-// other path costs them no registers).
-template <class V, int FIELD = 2>
-__device__ __forceinline__ Porous<V> porous_at(const Phys<V> &p, int64_t k)
+// other path costs them no registers).  k: the node's offset in a plane, or
+// the Darcy number itself where a kernel has loaded it.
+template <class V>
+struct Darcy {
+    V da;
+};
+template <class V>
+__device__ __forceinline__ V darcy_of(const Phys<V> &p, int64_t k) { return load_da(p, k); }
+template <class V>
+__device__ __forceinline__ V darcy_of(const Phys<V> &, Darcy<V> d) { return d.da; }
+template <class V, int FIELD = 2, class K = int64_t>
+__device__ __forceinline__ Porous<V> porous_at(const Phys<V> &p, K k)
 {
     Porous<V> q;
     if (FIELD == 0 || (FIELD == 2 && !p.da)) {
@@ -580,7 +622,7 @@ __device__ __forceinline__ Porous<V> porous_at(const Phys<V> &p, int64_t k)
         q.eFsK = p.eFe_isqK;
         return q;
     }
-    const V iK = vrcp(load_da(p, k) * p.L2);
+    const V iK = vrcp(darcy_of(p, k) * p.L2);
     const V isK = vsqrt(iK);
     q.heK = V(0.25) * p.eps * iK;
     q.eK = p.eps * iK;
@@ -598,8 +640,8 @@ __device__ __forceinline__ Porous<V> porous_at(const Phys<V> &p, int64_t k)
 // DEV = 1: f and g are deviations from the rest state (f_i - w_i,
 // g_i - w_i T_m), so the zeroth moments are rho - 1 and T - T_m; every other
 // moment used is the same linear form of the deviations.
-template <class V, int FIELD = 2, int DEV = 0>
-__device__ __forceinline__ Macro<V> macro(const Phys<V> &p, const V f[9], const V g[5], V tau_prev, int64_t k)
+template <class V, int FIELD = 2, int DEV = 0, class K = int64_t>
+__device__ __forceinline__ Macro<V> macro(const Phys<V> &p, const V f[9], const V g[5], V tau_prev, K k)
 {
     Macro<V> m;
     const Porous<V> q = porous_at<V, FIELD>(p, k);
@@ -682,8 +724,8 @@ __device__ __forceinline__ F2 tau_newton(const Phys<F2> &p, F2 tau, F2 gs, F2 bc
               tau_newton_s(tau.v.y, gs.v.y, bc.v.y, ss.v.y, g1, g2, nm1, Dhi, p.clamp_mode, nu3));
 }
 
-template <class V, int FIELD = 2, int DEV = 0>
-__device__ __forceinline__ V implicit_tau(const Phys<V> &p, const V f[9], const V g[5], int64_t k)
+template <class V, int FIELD = 2, int DEV = 0, class K = int64_t, class Z = AsUsual>
+__device__ __forceinline__ V implicit_tau(const Phys<V> &p, const V f[9], const V g[5], K k, Z z = Z())
 {
     const Porous<V> q = porous_at<V, FIELD>(p, k);
     // moments that do not depend on tau (as in macro() and collide(); DEV as
@@ -716,8 +758,8 @@ __device__ __forceinline__ V implicit_tau(const Phys<V> &p, const V f[9], const 
         const V e_eq = vfma(rho, u2e3, V(-2) * (DEV ? r0 : rho));
         const V w = vrcp(tau);
         const V A = V(1.4 / 6.0) * (e - e_eq);
-        const V B = V(0.5) * w * (pxx - rie * vfma(ux, ux, -(uy * uy)));
-        const V C = w * (pxy - rie * (ux * uy));
+        const V B = V(0.5) * w * nmad(rie, vfma(ux, ux, -(uy * uy)), pxx, z);
+        const V C = w * nmad(rie, ux * uy, pxy, z);
         const V bc = vfma(B, B, C * C);
         const V ss = vfma(A, A, bc);
         tau = tau_newton(p, tau, gsc * vsqrt(ss), bc, ss);
@@ -727,11 +769,11 @@ __device__ __forceinline__ V implicit_tau(const Phys<V> &p, const V f[9], const 
 
 // tau the collision of a node starts from: TAU 0 the stored lagged value
 // (loaded only then), TAU 1 the implicit solve.
-template <int TAU, class V, int FIELD, int DEV = 0, class Load>
-__device__ __forceinline__ V tau_start(const Phys<V> &p, const V f[9], const V g[5], int64_t k, Load load)
+template <int TAU, class V, int FIELD, int DEV = 0, class Load, class K = int64_t, class Z = AsUsual>
+__device__ __forceinline__ V tau_start(const Phys<V> &p, const V f[9], const V g[5], K k, Load load, Z z = Z())
 {
     if constexpr (TAU == 1)
-        return implicit_tau<V, FIELD, DEV>(p, f, g, k);
+        return implicit_tau<V, FIELD, DEV>(p, f, g, k, z);
     else
         return load();
 }
@@ -739,9 +781,10 @@ __device__ __forceinline__ V tau_start(const Phys<V> &p, const V f[9], const V g
 // Full node update in place: f, g become the post-collision populations.
 // Returns the new relaxation time; m receives the macroscopic moments and the
 // apparent lattice viscosity of this collision.  k is the node's offset in a
-// plane (used only to read a per-node Darcy field).
-template <class V, int FIELD = 2, int DEV = 0>
-__device__ __forceinline__ V collide(const Phys<V> &p, V f[9], V g[5], V tau_prev, Macro<V> &m, int64_t k)
+// plane, or its Darcy number (used only with a per-node Darcy field); z: how
+// single nodes among a pair are rounded (above).
+template <class V, int FIELD = 2, int DEV = 0, class K = int64_t, class Z = AsUsual>
+__device__ __forceinline__ V collide(const Phys<V> &p, V f[9], V g[5], V tau_prev, Macro<V> &m, K k, Z z = Z())
 {
     m = macro<V, FIELD, DEV>(p, f, g, tau_prev, k);
     const V rho = m.rho, ux = m.ux, uy = m.uy;
@@ -761,16 +804,16 @@ __device__ __forceinline__ V collide(const Phys<V> &p, V f[9], V g[5], V tau_pre
     const V r0 = DEV ? m.drho : rho;
     const V e_eq = vfma(rho, u2e3, V(-2) * r0);
     const V ep_eq = r0 - rho * u2e3;
-    const V pxx_eq = rie * vfma(ux, ux, -(uy * uy));
-    const V pxy_eq = rie * (ux * uy);
+    const V pxx_neq = nmad(rie, vfma(ux, ux, -(uy * uy)), pxx, z);
+    const V pxy_neq = nmad(rie, ux * uy, pxy, z);
     // strain rate from the non-equilibrium moments with the lagged tau:
     // gamma_xx,yy = -3/(2 rho) (s1 e_neq / 6 +- w pxx_neq / 2),
     // gamma_xy = -3/(2 rho) w pxy_neq, |gamma| = sqrt(2 gamma:gamma)
     //          = (3 / rho) sqrt(A^2 + B^2 + C^2)
     const V wp = vrcp(tau_prev);
     const V A = V(1.4 / 6.0) * (e - e_eq);
-    const V B = V(0.5) * wp * (pxx - pxx_eq);
-    const V C = wp * (pxy - pxy_eq);
+    const V B = V(0.5) * wp * pxx_neq;
+    const V C = wp * pxy_neq;
     const V gam = V(3) * m.irho * vsqrt(vfma(A, A, vfma(B, B, C * C)));
     const V nu = p.nu_ref * apparent<V>(p, gam * p.gamma_scale);
     const V tau = vfma(V(3), nu, V(0.5));
@@ -788,8 +831,8 @@ __device__ __forceinline__ V collide(const Phys<V> &p, V f[9], V g[5], V tau_pre
     const V qxs = vfma(V(-0.4) * rho, m.Fx, vfma(V(-1.2), vfma(rho, ux, qx), qx));
     const V qys = vfma(V(-0.4) * rho, m.Fy, vfma(V(-1.2), vfma(rho, uy, qy), qy));
     const V hw = vfma(V(-0.5), w, V(1));
-    const V pxxs = vfma(hw, Fxx, vfma(-w, pxx - pxx_eq, pxx));
-    const V pxys = vfma(hw, Fxy, vfma(-w, pxy - pxy_eq, pxy));
+    const V pxxs = vfma(hw, Fxx, vfma(-w, pxx_neq, pxx));
+    const V pxys = vfma(hw, Fxy, vfma(-w, pxy_neq, pxy));
     // f* = M^T diag(1/9, 1/36, 1/36, 1/6, 1/12, 1/6, 1/12, 1/4, 1/4) m*
     const V a0 = r0 * V(1.0 / 9.0), a1 = es * V(1.0 / 36.0), a2 = eps_s * V(1.0 / 36.0);
     const V a3 = jxs * V(1.0 / 6.0), a4 = qxs * V(1.0 / 12.0);
@@ -819,9 +862,9 @@ __device__ __forceinline__ V collide(const Phys<V> &p, V f[9], V g[5], V tau_pre
     const V n3s = vfma(-p.s_e, vfma(V(2.0 / 3.0), T0, n3), n3);
     const V n4s = vfma(-p.s_p, n4, n4);
     // g* = N^T diag(1/5, 1/2, 1/2, 1/20, 1/4) n*
-    const V t0 = T0 * V(0.2), t3 = n3s * V(0.05), t4 = n4s * V(0.25);
+    const V t0 = T0 * V(0.2), t4 = n4s * V(0.25);
     const V h1 = n1s * V(0.5), h2 = n2s * V(0.5);
-    const V t03 = t0 + t3;
+    const V t03 = pmad(n3s, V(0.05), t0, z);
     g[0] = vfma(V(-0.2), n3s, t0);
     g[1] = t03 + h1 + t4;
     g[2] = t03 + h2 - t4;

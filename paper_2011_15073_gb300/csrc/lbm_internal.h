@@ -75,6 +75,10 @@ namespace lbm {
 // cudaError_t from cudaGetLastError().
 cudaError_t launch_init(lbm_ctx *c);
 cudaError_t launch_step(lbm_ctx *c);
+// Two steps in one launch (lbm_strip.cu), the same values as two launch_step
+// calls bit for bit, where two_steps() says that it pays.
+bool two_steps(const lbm_ctx *c);
+cudaError_t launch_two_steps(lbm_ctx *c);
 // Write the context's step count to d_step_base (before a step-graph replay).
 cudaError_t launch_set_step_base(lbm_ctx *c);
 // One step of the two-buffer layout between explicit state buffers (same

@@ -1,0 +1,47 @@
+"""Two time steps in one launch (csrc/lbm_strip.cu): the FP32 storages' step()
+of several steps takes that kernel on large grids, single steps never do, and
+both give the same state bit for bit -- the walls, the columns the one-step
+kernel updates one node at a time, odd widths, and every place at which strips
+and their segments can end."""
+import numpy as np
+import pytest
+
+from paper_2011_15073_gb300 import inputs, lbm
+
+pytestmark = pytest.mark.gpu
+
+
+def state_after(nx, ny, parts, field, **opts):
+    with lbm.Cavity(nx, ny, 0.7, 1e-2, 1e5, 6.2, 0.6, **opts) as c:
+        if field:
+            c.set_darcy_field(inputs.darcy_field(1, nx, ny))
+        c.set_state_f64(*inputs.perturbed_state(c.get_state_f64(), seed=nx + ny, amp=1e-2))
+        for k in parts:
+            c.step(k)
+        host = np.empty(c.state_bytes(), np.uint8)
+        c.get_state(host)
+        assert lbm.debug_padding_canary(c.ctx) == 0
+    # with the implicit tau the tau plane is no state
+    return host[:14 * nx * ny * 4] if opts.get("tau_iters") else host
+
+
+# 600,000 nodes (2,000,000 with the implicit tau) or more take the kernel; the
+# widths put the right wall at every offset class of the 60-column strips and
+# the 64-column tiles, the smallest and tallest grids end the segments' range
+@pytest.mark.parametrize("nx,ny,opts", [
+    (1024, 600, dict(prec="f32d")), (1021, 613, dict(prec="f32")), (961, 640, dict(prec="f32d", clamp_mode=1)),
+    (1022, 600, dict(prec="f32")), (128, 4700, dict(prec="f32d")), (129, 4800, dict(prec="f32", clamp_mode=1)),
+    (9600, 64, dict(prec="f32d")), (1500, 1400, dict(prec="f32", tau_iters=2, clamp_mode=1)),
+    (1501, 1403, dict(prec="f32d", tau_iters=1))])
+@pytest.mark.parametrize("field", [False, True])
+def test_equals_single_steps_bit_for_bit(nx, ny, opts, field):
+    one = state_after(nx, ny, [1] * 21, field, **opts)
+    two = state_after(nx, ny, [7, 14], field, **opts)
+    assert np.array_equal(one, two)
+
+
+def test_in_replayed_graphs():
+    """Graphs of double steps: lengths that are no multiple of four, and odd remainders."""
+    one = state_after(1024, 600, [1] * 31, False, prec="f32d")
+    for g in (2, 6, 8):
+        assert np.array_equal(one, state_after(1024, 600, [11, 20], False, prec="f32d", graph_steps=g))
