@@ -59,8 +59,10 @@ __device__ __forceinline__ F2 vfma(F2 a, F2 b, F2 c) { return F2(__ffma2_rn(a.v,
 // them, the packed ones round the product first, and a node's rounding must not
 // depend on the kernel that updates it: FP32 runs are compared bit for bit
 // between kernels.  So a packed kernel that takes wall nodes too says which
-// components of its pair are to be rounded as single nodes (SingleLanes).
+// components of its pair are to be rounded as single nodes (SingleLanes), or
+// that both are (AsSingle).
 struct AsUsual {};
+struct AsSingle {};
 struct SingleLanes {
     bool x, y;
 };
@@ -73,10 +75,12 @@ __device__ __forceinline__ F2 nmad(F2 a, F2 b, F2 c, SingleLanes z)
     const F2 two = c - a * b, one = vfma(-a, b, c);
     return F2(z.x ? one.v.x : two.v.x, z.y ? one.v.y : two.v.y);
 }
+__device__ __forceinline__ F2 nmad(F2 a, F2 b, F2 c, AsSingle) { return vfma(-a, b, c); }
 // c + a b
 __device__ __forceinline__ double pmad(double a, double b, double c, AsUsual) { return c + a * b; }
 __device__ __forceinline__ float pmad(float a, float b, float c, AsUsual) { return fmaf(a, b, c); }
 __device__ __forceinline__ F2 pmad(F2 a, F2 b, F2 c, AsUsual) { return c + a * b; }
+__device__ __forceinline__ F2 pmad(F2 a, F2 b, F2 c, AsSingle) { return vfma(a, b, c); }
 __device__ __forceinline__ F2 pmad(F2 a, F2 b, F2 c, SingleLanes z)
 {
     const F2 two = c + a * b, one = vfma(a, b, c);

@@ -39,16 +39,59 @@ __device__ __forceinline__ void step_node(const typename Store<PREC>::S *__restr
     if constexpr (TAU == 0) tdst[k] = typename St::TauS(tau);
 }
 
+// A pair of nodes (x0, x0 + 1) of a row with the wall rules: each node's
+// populations pulled on their own, both collided as one packed pair, rounded
+// as single nodes.  One at a time, as the 16-bit storages and the implicit tau
+// still do, the second node's loads and arithmetic follow the first's: 128^2
+// (all warps touch a wall) 2.38 -> 1.99 us per step, 256^2 (half of them) 3.05
+// -> 2.58, 512^2 5.2 -> 4.8.  With the implicit tau the second collision costs
+// registers that its grids miss more (1200^2 35.0 -> 36.4 us).
+template <int PREC, int FIELD, int TAU>
+__device__ __forceinline__ void step2_walls(const typename Store<PREC>::S *__restrict__ src,
+                                            typename Store<PREC>::S *__restrict__ dst,
+                                            const float *__restrict__ tsrc, float *__restrict__ tdst,
+                                            const Phys<float> &p, const Phys<F2> &p2, int x0, int y)
+{
+    using St = Store<PREC>;
+    const bool two = x0 + 1 < p.nx;
+    const int64_t P = p.plane, k = (int64_t)y * p.pitch + x0;
+    float fa[9], ga[5], fb[9], gb[5];
+    pull<PREC, float, false, 1>(src, p, x0, y, fa, ga);
+    pull<PREC, float, false, 1>(src, p, two ? x0 + 1 : x0, y, fb, gb);
+    F2 f[9], g[5];
+#pragma unroll
+    for (int i = 0; i < 9; i++) f[i] = F2(fa[i], fb[i]);
+#pragma unroll
+    for (int i = 0; i < 5; i++) g[i] = F2(ga[i], gb[i]);
+    // an odd row's last pair reads one element of the row's padding here
+    const F2 t0 = tau_start<TAU, F2, FIELD, 1>(p2, f, g, k, [&] { return F2(*reinterpret_cast<const float2 *>(tsrc + k)); },
+                                               AsSingle{});
+    Macro<F2> m;
+    const F2 tau = collide<F2, FIELD, 1>(p2, f, g, t0, m, k, AsSingle{});
+    uint32_t rng = 0;
+    if (two) {
+#pragma unroll
+        for (int i = 0; i < 9; i++) St::sdv2(dst + i * P, k, f[i], float(rest_f(i)), rng);
+#pragma unroll
+        for (int i = 0; i < 5; i++) St::sdv2(dst + (9 + i) * P, k, g[i], float(rest_g(i)), rng);
+        if constexpr (TAU == 0) *reinterpret_cast<float2 *>(tdst + k) = tau.v;
+    } else {
+#pragma unroll
+        for (int i = 0; i < 9; i++) St::sdv(dst + i * P, k, f[i].v.x, float(rest_f(i)), rng);
+#pragma unroll
+        for (int i = 0; i < 5; i++) St::sdv(dst + (9 + i) * P, k, g[i].v.x, float(rest_g(i)), rng);
+        if constexpr (TAU == 0) tdst[k] = tau.v.x;
+    }
+}
+
 // One tile of a row: thread t of the block updates nodes xbase + 2t and
 // xbase + 2t + 1 of row y.  A warp whose 64 nodes and their neighbours are
 // all interior takes the fast path -- aligned pair loads and stores, the
 // x-shifted populations exchanged by warp shuffles, both nodes' arithmetic
 // on the packed FP32x2 pipe; any warp that touches a wall or the ragged end
-// of a row updates its nodes one at a time with the wall rules.  The branch
-// is uniform per warp.  (Handing the side-wall warps to the packed path, as
-// step4_tile does, costs this tile 8-40 registers per thread in its
-// single-cavity and batched kernels; at 64 nodes per warp the wall warps are
-// a small share of a row.)  TAU and seed as for step_node.
+// of a row takes the wall rules (step2_walls, or one node at a time with the
+// 16-bit storages and the implicit tau).  The branch is uniform per warp.  TAU and seed as for
+// step_node.
 template <int PREC, int FIELD = 2, int TAU = 0>
 __device__ __forceinline__ void step2_tile(const typename Store<PREC>::S *__restrict__ src,
                                            typename Store<PREC>::S *__restrict__ dst,
@@ -63,6 +106,10 @@ __device__ __forceinline__ void step2_tile(const typename Store<PREC>::S *__rest
     const int wx = xbase + 2 * (threadIdx.x & ~31);
     const bool fast = y > 0 && y < p.ny - 1 && wx > 0 && wx + 64 < p.nx;
     if (!fast) {
+        if constexpr (!is16<PREC>() && TAU == 0) {
+            if (x0 < p.nx) step2_walls<PREC, FIELD, TAU>(src, dst, tsrc, tdst, p, p2, x0, y);
+            return;
+        }
         for (int j = 0; j < 2; j++)
             if (x0 + j < p.nx) step_node<PREC, float, FIELD, TAU>(src, dst, tsrc, tdst, p, x0 + j, y, seed);
         return;
