@@ -117,9 +117,10 @@ typedef struct {
                           walls) differ between modes               [0]    */
     int graph_steps;   /* lbm_step replays a CUDA graph of this many
                           steps (rounded up to even) instead of one
-                          launch per step, which pays on small,
-                          launch-bound grids: 0 auto (64 steps for
-                          grids of at most 512 x 512 nodes, none for
+                          launch after the other, which pays on small and
+                          middle-sized grids, bound by launches: 0 auto
+                          (64 steps for grids of at most 2,000,000 nodes,
+                          none for
                           F16S / BF16S in layout 1), -1 never, G > 0
                           always (F16S / BF16S with layout 1 get
                           LBM_ERR_UNSUPPORTED).  With F16S / BF16S the
@@ -186,7 +187,9 @@ int lbm_set_darcy_field(lbm_ctx *ctx, const double *Da_xy);
 /* Copy the lattice-unit parameters of ctx into *out. */
 int lbm_get_lattice(const lbm_ctx *ctx, lbm_lattice *out);
 
-/* Advance k >= 0 time steps.  Each step is one launch of the fused kernel:
+/* Advance k >= 0 time steps.  Each step, or on large grids with FP32 storage
+ * each pair of steps, is one launch of the fused kernel (the values are the
+ * same either way):
  * pull streaming with the wall rules, macroscopic moments (Eqs.
  * macro_fluid_density, velo), porous velocity solve, strain rate from the
  * non-equilibrium moments and the modified power law (Eq. MPL and the

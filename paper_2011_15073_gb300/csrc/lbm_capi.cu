@@ -42,7 +42,11 @@ int graph_len_for(const lbm_ctx *c)
     // the stochastic-rounding storages take their seeds from the device in a
     // graph: built for the two-buffer kernels, not the in-place ones
     const bool sr_aa = lbm::rounds_stochastically(c->opts.prec) && c->opts.layout == 1;
-    return (!sr_aa && (int64_t)c->nx * c->ny <= 512 * 512) ? 64 : 0;
+    // Up to here a replay is faster than launch after launch by more than 1 us
+    // per kernel: 701 x 499 8.2 -> 6.0 us per step, 1024 x 512 10.3 -> 7.1, 1024^2
+    // (two steps per launch) 15.5 -> 14.4, 1200^2 with the implicit tau 36.5 ->
+    // 34.6.
+    return (!sr_aa && (int64_t)c->nx * c->ny <= 2000000) ? 64 : 0;
 }
 
 int graph_parity(const lbm_ctx *c) { return c->opts.layout == 1 ? (c->aa_form_o ? 1 : 0) : c->cur; }
