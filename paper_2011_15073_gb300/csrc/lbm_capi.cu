@@ -51,6 +51,19 @@ int graph_len_for(const lbm_ctx *c)
 
 int graph_parity(const lbm_ctx *c) { return c->opts.layout == 1 ? (c->aa_form_o ? 1 : 0) : c->cur; }
 
+// Steps that one launch takes where several are due (1: one).
+int steps_per_launch(const lbm_ctx *c)
+{
+    if (lbm::two_steps(c)) return 2;
+    const int m = lbm::tile_steps(c);
+    return m > 1 ? m : 1;
+}
+// m = 1, or a number of steps up to steps_per_launch() that a launch can take
+cudaError_t launch_steps(lbm_ctx *c, int m)
+{
+    return m == 1 ? lbm::launch_step(c) : (lbm::two_steps(c) ? lbm::launch_two_steps(c) : lbm::launch_tile(c, m));
+}
+
 // Capture G step launches on the context's stream into an executable graph
 // for the current parity.  Launching records nothing while capturing, and G
 // is even, so the buffer state is back where it started afterwards.
@@ -69,11 +82,11 @@ int capture_steps(lbm_ctx *c, int G, int par)
     cudaError_t e = cudaSuccess;
     const bool sr = lbm::rounds_stochastically(c->opts.prec);
     int i = 0;
-    // an even number of double steps, so that they too end in the buffer they began in
-    if (lbm::two_steps(c))
-        for (; i + 4 <= G && e == cudaSuccess; i += 4) {
-            e = lbm::launch_two_steps(c);
-            if (e == cudaSuccess) e = lbm::launch_two_steps(c);
+    // an even number of such launches, so that they too end in the buffer they began in
+    if (const int m = steps_per_launch(c); m > 1)
+        for (; i + 2 * m <= G && e == cudaSuccess; i += 2 * m) {
+            e = launch_steps(c, m);
+            if (e == cudaSuccess) e = launch_steps(c, m);
         }
     for (; i < G && e == cudaSuccess; i++) {
         c->capture_s = sr ? i : -1;   // seeds from d_step_base + i (lbm_kernels.cu)
@@ -493,14 +506,9 @@ int lbm_step(lbm_ctx *c, int64_t k)
             t += G;
         }
     }
-    if (lbm::two_steps(c))
-        for (; t + 2 <= k; t += 2) {
-            CK(lbm::launch_two_steps(c));
-            c->steps += 2;
-        }
-    for (; t < k; t++) {
-        CK(lbm::launch_step(c));
-        c->steps++;   // also the stochastic rounding's step counter
+    for (int m = steps_per_launch(c); t < k; t += m, c->steps += m) {   // also the stochastic rounding's step counter
+        while (m > k - t) m /= 2;   // 4, 2, 1
+        CK(launch_steps(c, m));
     }
     return LBM_OK;
 }

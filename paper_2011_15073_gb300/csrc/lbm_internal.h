@@ -75,10 +75,13 @@ namespace lbm {
 // cudaError_t from cudaGetLastError().
 cudaError_t launch_init(lbm_ctx *c);
 cudaError_t launch_step(lbm_ctx *c);
-// Two steps in one launch (lbm_strip.cu), the same values as two launch_step
-// calls bit for bit, where two_steps() says that it pays.
+// Several steps in one launch, the same values as launch_step calls bit for
+// bit: two on large grids (lbm_strip.cu) where two_steps() says that it pays,
+// two or four on small ones (lbm_tile.cu) where tile_steps() does (0: not).
 bool two_steps(const lbm_ctx *c);
 cudaError_t launch_two_steps(lbm_ctx *c);
+int tile_steps(const lbm_ctx *c);
+cudaError_t launch_tile(lbm_ctx *c, int steps);
 // Write the context's step count to d_step_base (before a step-graph replay).
 cudaError_t launch_set_step_base(lbm_ctx *c);
 // One step of the two-buffer layout between explicit state buffers (same

@@ -1,8 +1,9 @@
-"""Two time steps in one launch (csrc/lbm_strip.cu): the FP32 storages' step()
-of several steps takes that kernel on large grids, single steps never do, and
-both give the same state bit for bit -- the walls, the columns the one-step
-kernel updates one node at a time, odd widths, and every place at which strips
-and their segments can end."""
+"""Several time steps in one launch (csrc/lbm_strip.cu on large grids, two at a
+time; csrc/lbm_tile.cu on small ones, four or two): the FP32 storages' step() of
+several steps takes these kernels, single steps never do, and both give the same
+state bit for bit -- the walls, the columns the one-step kernel updates one node
+at a time, odd widths, and every place at which strips and their segments, or
+the windows, can end."""
 import numpy as np
 import pytest
 
@@ -45,3 +46,18 @@ def test_in_replayed_graphs():
     one = state_after(1024, 600, [1] * 31, False, prec="f32d")
     for g in (2, 6, 8):
         assert np.array_equal(one, state_after(1024, 600, [11, 20], False, prec="f32d", graph_steps=g))
+
+
+# at most 152 windows of 56 x 10 nodes (four steps) or 60 x 14 (two); widths and
+# heights one more and one less than whole windows, the walls on the windows'
+# first and last columns, the smallest width that takes the kernel
+@pytest.mark.parametrize("nx,ny,opts", [
+    (64, 2, dict(prec="f32d")), (65, 65, dict(prec="f32")), (112, 20, dict(prec="f32d", clamp_mode=1)),
+    (113, 21, dict(prec="f32")), (111, 19, dict(prec="f32d")), (191, 64, dict(prec="f32d")),
+    (256, 256, dict(prec="f32d", tau_iters=2)), (129, 301, dict(prec="f32", tau_iters=1, clamp_mode=1)),
+    (300, 300, dict(prec="f32d")), (301, 281, dict(prec="f32"))])
+@pytest.mark.parametrize("field", [False, True])
+def test_small_grids_equal_single_steps_bit_for_bit(nx, ny, opts, field):
+    one = state_after(nx, ny, [1] * 83, field, **opts)
+    many = state_after(nx, ny, [7, 76], field, **opts)   # 4 + 2 + 1, and a replayed graph
+    assert np.array_equal(one, many)
