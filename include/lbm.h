@@ -321,7 +321,9 @@ void lbm_batch_destroy(lbm_batch *batch);
 /* Borrow case i's context for state I/O, fields or Nu (do not destroy it). */
 int lbm_batch_get_case(lbm_batch *batch, int i, lbm_ctx **ctx);
 
-/* Advance every case k steps (one launch per step). Asynchronous. */
+/* Advance every case k steps (one launch per step of the plan below, or with
+ * FP32 storage and many nodes per two steps; the values are the same).
+ * Asynchronous. */
 int lbm_batch_step(lbm_batch *batch, int64_t k);
 
 /* Run every case until its residual (as lbm_run_to_steady) falls below tol,

@@ -19,6 +19,7 @@
 #include "lbm_internal.h"
 #include "lbm_trace.h"
 #include "lbm_step.cuh"
+#include "lbm_strip.cuh"
 
 namespace {
 
@@ -46,12 +47,23 @@ struct Conv {
 };
 
 // The compacted list of active cases: idx[0..m) the active cases in order,
-// t0[j] the first flat tile of idx[j] (t0[m] = total), hdr = {m, total}.
+// t0[j] the first flat tile of idx[j] (t0[m] = total), u0[j] its first unit
+// of the two-step strips (lbm_strip.cuh), hdr = {m, tiles, units, rows per
+// unit}.  slots: the warps of the two-step kernel that fit on the chip.
 struct ActiveList {
     int *idx;
     int *t0;
+    int *u0;
     int *hdr;
+    int slots;
 };
+// The strips of a case whose units have about `rows` rows each.
+__device__ __forceinline__ StripPlan case_plan(const CaseDev &c, int rows)
+{
+    StripPlan plan = strip_plan(c.pf.nx);
+    plan.cut(c.pf.ny, c.pf.ny / rows);
+    return plan;
+}
 
 // Grid barrier of the persistent kernel: arrival count and generation.
 struct GridBarrier {
@@ -73,6 +85,18 @@ __device__ void build_active(const CaseDev *cases, const int *active, int n, Act
     a.t0[m] = t;
     a.hdr[0] = m;
     a.hdr[1] = t;
+    // rows per unit for about as many units as warps fit on the chip
+    long long weight = 0;
+    for (int j = 0; j < m; j++) weight += strip_plan(cases[a.idx[j]].pf.nx).weight(cases[a.idx[j]].pf.ny);
+    const long long rows = (weight + 2 * a.slots - 1) / (2 * a.slots);
+    a.hdr[3] = rows > 4 ? (int)rows : 4;
+    int u = 0;
+    for (int j = 0; j < m; j++) {
+        a.u0[j] = u;
+        u += case_plan(cases[a.idx[j]], a.hdr[3]).units();
+    }
+    a.u0[m] = u;
+    a.hdr[2] = u;
 }
 
 __global__ void build_active_kernel(const CaseDev *cases, const int *active, int n, ActiveList a)
@@ -141,6 +165,38 @@ __global__ void __launch_bounds__(256)
 batch_step_kernel(const CaseDev *__restrict__ cases, ActiveList a, StepAt at)
 {
     batch_sweep<PREC, TAU, FIELD>(cases, a, a.hdr[0], a.hdr[1], at);
+}
+
+// Two steps of every active case in one launch, strip unit by strip unit
+// (lbm_strip.cuh): half the HBM traffic of the tile sweep.  odd: an odd number
+// of such launches has run since the cases were uploaded.  The unit's case
+// constants are copied to shared memory (in the single-cavity kernel they are
+// launch parameters).
+template <int PREC, int TAU>
+__global__ void __launch_bounds__(32, strip_blocks<TAU>())
+batch_strip_kernel(const CaseDev *__restrict__ cases, ActiveList a, int odd)
+{
+    using S = typename Store<PREC>::S;
+    __shared__ S ring[3][14][64];
+    __shared__ float tring[3][64];
+    __shared__ Phys<F2> p;
+    static_assert(sizeof(Phys<F2>) % 4 == 0, "copied word by word");
+    const int m = a.hdr[0], total = a.hdr[2], rows = a.hdr[3];
+    for (int u = blockIdx.x; u < total; u += gridDim.x) {
+        int lo = 0, hi = m - 1;
+        while (lo < hi) {
+            const int mid = (lo + hi + 1) >> 1;
+            if (a.u0[mid] <= u) lo = mid; else hi = mid - 1;
+        }
+        const CaseDev &cd = cases[a.idx[lo]];
+        __syncwarp();   // the unit before has read p
+        for (int w = threadIdx.x; w < (int)(sizeof(p) / 4); w += 32)
+            reinterpret_cast<uint32_t *>(&p)[w] = reinterpret_cast<const uint32_t *>(&cd.p2)[w];
+        __syncwarp();
+        const int s = cd.cur ^ odd;
+        strip_unit<PREC, 0, TAU>((const S *)cd.dist[s], (S *)cd.dist[s ^ 1], (const float *)cd.tau[s],
+                                 (float *)cd.tau[s ^ 1], p, case_plan(cd, rows), u - a.u0[lo], ring, tring);
+    }
 }
 
 // Bounded grid barrier.  Thread 0 of each block arrives on the counter; the
@@ -272,7 +328,7 @@ struct lbm_batch {
     std::vector<CaseDev> host_cases;
     CaseDev *d_cases = nullptr;
     int *d_active = nullptr;
-    ActiveList act{nullptr, nullptr, nullptr};
+    ActiveList act{nullptr, nullptr, nullptr, nullptr, 0};
     Conv *d_conv = nullptr;
     double **d_smalls = nullptr;
     int *d_chunks = nullptr;
@@ -384,6 +440,29 @@ cudaError_t launch_batch_step(lbm_batch *b, StepAt at)
     return cudaLaunchKernel(kernel_of(b, false), dim3(grid_blocks(b)), dim3(b->threads), args, 0, b->stream);
 }
 
+// Whether lbm_batch_step takes two steps per launch: FP32 storage without a
+// per-node Darcy field, and enough nodes to fill the chip (as two_steps() for
+// one cavity; the smallest widths share a lane between both side walls).
+bool batch_strips(const lbm_batch *b)
+{
+    if (b->any_field || (b->opts.prec != LBM_F32 && b->opts.prec != LBM_F32D) || b->opts.staging != 0) return false;
+    int64_t nodes = 0;
+    for (const lbm_ctx *c : b->sub) {
+        if (c->nx < 64 || c->ny < 16) return false;
+        nodes += (int64_t)c->nx * c->ny;
+    }
+    return nodes >= (b->opts.tau_iters > 0 ? 2000000 : 600000);
+}
+
+cudaError_t launch_batch_strips(lbm_batch *b, int odd)
+{
+    const bool implicit = b->opts.tau_iters > 0;
+    auto *kern = b->opts.prec == LBM_F32 ? (implicit ? batch_strip_kernel<LBM_F32, 1> : batch_strip_kernel<LBM_F32, 0>)
+                                         : (implicit ? batch_strip_kernel<LBM_F32D, 1> : batch_strip_kernel<LBM_F32D, 0>);
+    kern<<<b->act.slots, 32, 0, b->stream>>>(b->d_cases, b->act, odd);
+    return cudaGetLastError();
+}
+
 // `steps` steps of every active case, `off` steps into the batch call (and
 // counted from the convergence records in a run to steady state): per-step
 // launches, or one persistent cooperative launch (its barrier reset first).
@@ -458,6 +537,7 @@ void free_batch(lbm_batch *b)
     cudaFree(b->d_active);
     cudaFree(b->act.idx);
     cudaFree(b->act.t0);
+    cudaFree(b->act.u0);
     cudaFree(b->act.hdr);
     cudaFree(b->d_conv);
     cudaFree(b->d_smalls);
@@ -538,13 +618,15 @@ int lbm_batch_create(lbm_batch **out, const lbm_case *cases, int ncases, const l
             BK(cudaMemset(b->d_active, 0, sizeof(int) * n));
             BK(cudaMalloc(&b->act.idx, sizeof(int) * n));
             BK(cudaMalloc(&b->act.t0, sizeof(int) * (n + 1)));
-            BK(cudaMalloc(&b->act.hdr, sizeof(int) * 2));
+            BK(cudaMalloc(&b->act.u0, sizeof(int) * (n + 1)));
+            BK(cudaMalloc(&b->act.hdr, sizeof(int) * 4));
             BK(cudaMalloc(&b->d_bar, sizeof(GridBarrier)));
             BK(cudaMalloc(&b->d_err, sizeof(int)));
             BK(cudaMemset(b->d_err, 0, sizeof(int)));
             BK(cudaMallocHost(&b->h_err, sizeof(int)));
             *b->h_err = 0;
             BK(cudaDeviceGetAttribute(&b->sms, cudaDevAttrMultiProcessorCount, b->device));
+            b->act.slots = b->sms * (o.tau_iters > 0 ? strip_blocks<1>() : strip_blocks<0>());
             BK(cudaMalloc(&b->d_conv, sizeof(Conv) * n));
             BK(cudaMalloc(&b->d_smalls, sizeof(double *) * n));
             BK(cudaMalloc(&b->d_chunks, sizeof(int)));
@@ -590,7 +672,17 @@ int lbm_batch_step(lbm_batch *b, int64_t k)
     // in pieces of an even number of steps (each case then ends a piece in
     // the buffer it started it in), then the odd remainder
     const int64_t piece = 1 << 20;
-    for (int64_t done = 0; done < k;) {
+    int64_t done = 0;
+    if (batch_strips(b)) {
+        for (; k - done >= 2; done += 2) BK(launch_batch_strips(b, (int)(done >> 1) & 1));
+        if ((done >> 1) & 1)
+            for (lbm_ctx *c : b->sub) c->cur ^= 1;
+        if (done < k) {
+            rc = upload_cases(b);
+            if (rc) return rc;
+        }
+    }
+    while (done < k) {
         int64_t n = k - done < piece ? k - done : piece;
         if (n > 1) n &= ~int64_t(1);
         BK(launch_batch_steps(b, (int)n, done));

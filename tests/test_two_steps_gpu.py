@@ -61,3 +61,24 @@ def test_small_grids_equal_single_steps_bit_for_bit(nx, ny, opts, field):
     one = state_after(nx, ny, [1] * 83, field, **opts)
     many = state_after(nx, ny, [7, 76], field, **opts)   # 4 + 2 + 1, and a replayed graph
     assert np.array_equal(one, many)
+
+
+@pytest.mark.parametrize("opts", [dict(prec="f32d"), dict(prec="f32", clamp_mode=1), dict(prec="f32d", tau_iters=2)])
+def test_batches_equal_single_steps_bit_for_bit(opts):
+    """A batch large enough for two steps per launch: cavities of one strip and
+    of several, of few rows and many, in one list of units."""
+    grids = [(64, 16), (65, 301), (127, 130), (512, 512), (191, 77), (700, 499), (300, 300)]
+    if opts.get("tau_iters"):
+        grids += [(1024, 1024), (601, 603)]
+    cases = [dict(nx=a, ny=b, n=0.7, Da=1e-2, Ra=1e5, Pr=6.2, porosity=0.6) for a, b in grids]
+    with lbm.Batch(cases, **opts) as batch:
+        for i, (nx, ny) in enumerate(grids):
+            f, g, tau = lbm.get_state_f64(batch.case_ctx(i), nx, ny)
+            lbm.set_state_f64(batch.case_ctx(i), *inputs.perturbed_state((f, g, tau), seed=nx + ny, amp=1e-2))
+        for k in (7, 2, 12):
+            batch.step(k)
+        for i, (nx, ny) in enumerate(grids):
+            host = np.empty(lbm.state_bytes(batch.case_ctx(i)), np.uint8)
+            lbm.get_state(batch.case_ctx(i), host)
+            one = state_after(nx, ny, [1] * 21, False, **opts)
+            assert np.array_equal(one, host[:one.size]), (nx, ny)
