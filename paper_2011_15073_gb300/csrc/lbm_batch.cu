@@ -86,9 +86,9 @@ __device__ void build_active(const CaseDev *cases, const int *active, int n, Act
     a.hdr[0] = m;
     a.hdr[1] = t;
     // rows per unit for about as many units as warps fit on the chip
-    long long weight = 0;
-    for (int j = 0; j < m; j++) weight += strip_plan(cases[a.idx[j]].pf.nx).weight(cases[a.idx[j]].pf.ny);
-    const long long rows = (weight + 2 * a.slots - 1) / (2 * a.slots);
+    long long sum = 0;
+    for (int j = 0; j < m; j++) sum += (long long)strip_plan(cases[a.idx[j]].pf.nx).nstrips * cases[a.idx[j]].pf.ny;
+    const long long rows = (sum + a.slots - 1) / a.slots;
     a.hdr[3] = rows > 4 ? (int)rows : 4;
     int u = 0;
     for (int j = 0; j < m; j++) {

@@ -108,10 +108,10 @@ __device__ __forceinline__ void step2_tile(const typename Store<PREC>::S *__rest
     if (!fast) {
         if constexpr (!is16<PREC>() && TAU == 0) {
             if (x0 < p.nx) step2_walls<PREC, FIELD, TAU>(src, dst, tsrc, tdst, p, p2, x0, y);
-            return;
+        } else {
+            for (int j = 0; j < 2; j++)
+                if (x0 + j < p.nx) step_node<PREC, float, FIELD, TAU>(src, dst, tsrc, tdst, p, x0 + j, y, seed);
         }
-        for (int j = 0; j < 2; j++)
-            if (x0 + j < p.nx) step_node<PREC, float, FIELD, TAU>(src, dst, tsrc, tdst, p, x0 + j, y, seed);
         return;
     }
     const int64_t P = p.plane, W = p.pitch;

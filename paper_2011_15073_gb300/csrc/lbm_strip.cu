@@ -27,7 +27,7 @@ cudaError_t strip_tau(lbm_ctx *c)
     // implicit tau)
     const int slots = 152 * strip_blocks<TAU>() * (TAU == 1 ? 2 : 1);
     StripPlan plan = strip_plan(c->nx);
-    plan.cut(c->ny, 2ll * slots / (2 * plan.inner() + 3 * plan.edges()));
+    plan.cut(c->ny, slots / plan.nstrips);
     const int blocks = plan.units();
     auto *kern = c->d_da ? strip_kernel<PREC, 1, TAU> : strip_kernel<PREC, 0, TAU>;
     kern<<<blocks, 32, 0, c->stream>>>((const S *)c->buf.dist[s], (S *)c->buf.dist[d], (const float *)c->buf.tau[s],
@@ -44,8 +44,9 @@ cudaError_t strip_t(lbm_ctx *c)
 }  // namespace
 
 // Measured on the FP32 storages, one step per launch / two (us per step, lagged
-// tau): 701 x 499 8.2 / 8.2, 1024^2 20.5 / 15.4, 2048^2 77 / 48, 4096^2 290 /
-// 178; implicit tau: 2048^2 86 / 76.  Smaller grids have too few rows per warp:
+// tau): 701 x 499 6.2 / 8.2, 1024 x 640 about 9.0 / 9.4, 1024^2 20.5 / 13.8, 2048^2
+// 77 / 46, 4096^2 290 / 174; implicit tau: 2048^2 86 / 74.  Smaller grids stay in
+// L2 and have too few rows per warp:
 // a segment of four rows takes six rows' first steps, one after the other.
 // The 16-bit storages are bound by instruction issue, not by HBM, and keep
 // their four-node kernel.

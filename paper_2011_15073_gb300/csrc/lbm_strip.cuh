@@ -14,8 +14,8 @@
 // columns by shuffles, and each lane reads back only the ring columns that it
 // wrote.  The loads of row y + 1 are issued before row y is collided.
 //
-// Measured (4096^2, FP32 deviations): 290 -> 178 us per step, 94 G node
-// updates/s, 5.7 TB/s of DRAM traffic; instruction issue and the latency of
+// Measured (4096^2, FP32 deviations): 290 -> 174 us per step, 96 G node
+// updates/s, 5.8 TB/s of DRAM traffic; instruction issue and the latency of
 // the collision with 12 warps per SM bound it now.
 //
 // Every node gets the arithmetic, and so the bits, of the one-step kernel: the
@@ -30,8 +30,8 @@ namespace lbm {
 constexpr int kStripCols = 60;   // columns a warp brings to the second step
 
 // One-warp blocks per SM.  Lagged tau: 12, at up to 168 registers (4096^2
-// FP32 deviations 178 us per step; 13, 14 and 16, whose fewer registers leave
-// less room for the loads ahead, 211, 199 and 196).  The implicit tau waits
+// FP32 deviations 178 us per step when compared; 13, 14 and 16, whose fewer
+// registers leave less room for the loads ahead, 211, 199 and 196).  The implicit tau waits
 // for its special functions rather than for memory: 16, at up to 128 registers
 // (4096^2 FP32 281 against 323 us).
 template <int TAU>
@@ -40,24 +40,16 @@ constexpr int strip_blocks()
     return TAU == 1 ? 16 : 12;
 }
 
-// The strips and the row segments they are cut into, and the columns
-// [0, lo) and [hi, nx) which the one-step kernel updates one node at a time.
-// Strips [0, first) and [end, nstrips) hold such columns or a side wall; they
-// are cut into nedge segments, the others into nseg: half as many again,
-// because an edge strip's rows take longer (with equal segments its units end
-// last and the chip waits for them: 4096^2 194 against 178 us per step).
+// The strips, the row segments each is cut into, and the columns [0, lo) and
+// [hi, nx) which the one-step kernel updates one node at a time; strips
+// [0, first) and [end, nstrips) hold such columns or a side wall.
 struct StripPlan {
-    int nstrips, first, end, nseg, nedge, lo, hi;
-    __host__ __device__ int edges() const { return first + nstrips - end; }
-    __host__ __device__ int inner() const { return end - first; }
-    __host__ __device__ int units() const { return edges() * nedge + inner() * nseg; }
-    // the sum of the units' rows, in halves, if every unit had the same weight
-    __host__ __device__ long long weight(int ny) const { return (2ll * inner() + 3ll * edges()) * ny; }
+    int nstrips, first, end, nseg, lo, hi;
+    __host__ __device__ int units() const { return nstrips * nseg; }
     __host__ __device__ void cut(int ny, long long segments)
     {
-        const int most = ny / 4 > 1 ? ny / 4 : 1;
+        const int most = ny / 4 > 1 ? ny / 4 : 1;   // a segment also takes the first step of two rows beyond it
         nseg = segments < 1 ? 1 : (segments < most ? (int)segments : most);
-        nedge = 3 * nseg / 2 < most ? 3 * nseg / 2 : most;
     }
 };
 __host__ __device__ inline StripPlan strip_plan(int nx)
@@ -70,7 +62,7 @@ __host__ __device__ inline StripPlan strip_plan(int nx)
     s.first = (s.lo + 1) / kStripCols + 1;
     s.end = s.hi < 62 ? 0 : (s.hi - 62) / kStripCols + 1;
     if (s.end < s.first) s.end = s.first = s.nstrips;
-    s.nseg = s.nedge = 1;
+    s.nseg = 1;
     return s;
 }
 
@@ -81,11 +73,12 @@ __device__ __forceinline__ F2 pair_at(const typename Store<PREC>::S *p, int64_t 
     return Store<PREC>::ldd2(p, k, float(rest));
 }
 
-// Rows [ya, yb) of a strip brought to the second step by one warp.  EDGE: the
-// window holds a side wall or single-rounded columns, or the rows the bottom
-// or top wall; without it the loop has no wall rules at all, and no branch
-// around its loads, which would make the compiler wait for them there.
-template <int PREC, int FIELD, int TAU, bool EDGE>
+// Rows [ya, yb) of a strip brought to the second step by one warp.  SIDE: the
+// window holds a side wall or single-rounded columns; ROWS: the rows the
+// bottom or top wall.  Without them the loop has no wall rules at all; in no
+// form is there a branch around its loads, which would make the compiler wait
+// for them there.
+template <int PREC, int FIELD, int TAU, bool SIDE, bool ROWS>
 __device__ __forceinline__ void
 strip_rows(const typename Store<PREC>::S *__restrict__ src, typename Store<PREC>::S *__restrict__ dst,
            const float *__restrict__ tsrc, float *__restrict__ tdst, const Phys<F2> &p, int strip, int ya, int yb,
@@ -108,7 +101,9 @@ strip_rows(const typename Store<PREC>::S *__restrict__ src, typename Store<PREC>
     // top and bottom wall the populations that come back from the row itself
     Raw raw[14];
     F2 rawt, da;
-    float e0 = 0.f, e1 = 0.f;   // what comes back to a side wall's node from its own diagonals
+    // what comes back to a side wall's node from its own diagonals
+    S e0, e1;
+    const int64_t own0 = left ? 7 * P : 8 * P + right_y, own1 = left ? 6 * P : 5 * P + right_y;
     auto load = [&](int y) {
         const int64_t k = (int64_t)y * W + xc;
         const S *k0 = src + k;
@@ -119,37 +114,20 @@ strip_rows(const typename Store<PREC>::S *__restrict__ src, typename Store<PREC>
         get(9, 9 * P);
         get(10, 10 * P);
         get(12, 12 * P);
-        if (!EDGE || (y > 0 && y < ny - 1)) {
-            get(2, 2 * P - W);
-            get(4, 4 * P + W);
-            get(5, 5 * P - W);
-            get(6, 6 * P - W);
-            get(7, 7 * P + W);
-            get(8, 8 * P + W);
-            get(11, 11 * P - W);
-            get(13, 13 * P + W);
-        } else {
-            const bool below = y > 0, above = y < ny - 1;
-            get(2, below ? 2 * P - W : 4 * P);
-            get(4, above ? 4 * P + W : 2 * P);
-            get(5, below ? 5 * P - W : 7 * P);
-            get(6, below ? 6 * P - W : 8 * P);
-            get(7, above ? 7 * P + W : 5 * P);
-            get(8, above ? 8 * P + W : 6 * P);
-            get(11, below ? 11 * P - W : 13 * P);
-            get(13, above ? 13 * P + W : 11 * P);
-        }
+        const bool below = !ROWS || y > 0, above = !ROWS || y < ny - 1;
+        get(2, below ? 2 * P - W : 4 * P);
+        get(4, above ? 4 * P + W : 2 * P);
+        get(5, below ? 5 * P - W : 7 * P);
+        get(6, below ? 6 * P - W : 8 * P);
+        get(7, above ? 7 * P + W : 5 * P);
+        get(8, above ? 8 * P + W : 6 * P);
+        get(11, below ? 11 * P - W : 13 * P);
+        get(13, above ? 13 * P + W : 11 * P);
         if constexpr (TAU == 0) rawt = F2(*reinterpret_cast<const float2 *>(tsrc + k));
         if constexpr (FIELD == 1) da = load_da(p, k);
-        if constexpr (EDGE) {
-            if (left) {
-                e0 = St::ldd(k0 + 7 * P, 0, float(rest_f(7)));
-                e1 = St::ldd(k0 + 6 * P, 0, float(rest_f(6)));
-            }
-            if (right_x || right_y) {
-                e0 = St::ldd(k0 + 8 * P, right_y, float(rest_f(8)));
-                e1 = St::ldd(k0 + 5 * P, right_y, float(rest_f(5)));
-            }
+        if constexpr (SIDE) {   // every lane loads, the wall's lanes use it
+            e0 = k0[own0];
+            e1 = k0[own1];
         }
     };
     // the side walls' nodes: populations that come back from the node itself
@@ -185,8 +163,8 @@ strip_rows(const typename Store<PREC>::S *__restrict__ src, typename Store<PREC>
         }
     };
     auto update = [&](F2 f[9], F2 g[5], F2 t, F2 d, int y) {
-        if constexpr (EDGE) {
-            const bool one = single || y == 0 || y == ny - 1;
+        if constexpr (SIDE || ROWS) {
+            const bool one = single || (ROWS && (y == 0 || y == ny - 1));
             return update_as(f, g, t, d, SingleLanes{one, one});
         } else {
             return update_as(f, g, t, d, AsUsual{});
@@ -207,7 +185,7 @@ strip_rows(const typename Store<PREC>::S *__restrict__ src, typename Store<PREC>
         // instruction cache with the implicit tau
 #pragma unroll 1
         for (int step = 0; step < 2; step++) {
-            if (step == 0 ? EDGE && y > last : y <= ya) continue;
+            if (step == 0 ? ROWS && y > last : y <= ya) continue;
             const int Y = y - step;   // the row this step is taken on
             F2 f[9], g[5], t;
             if (step == 0) {
@@ -227,15 +205,20 @@ strip_rows(const typename Store<PREC>::S *__restrict__ src, typename Store<PREC>
                 g[2] = r_g(2);
                 g[3] = from_right(r_g(3), 0.f, lane);
                 g[4] = r_g(4);
-                if (EDGE && y == 0) {
+                if (ROWS && y == 0) {
                     f[5] = r_f(5);
                     f[6] = r_f(6);
                 }
-                if (EDGE && y == ny - 1) {
+                if (ROWS && y == ny - 1) {
                     f[7] = r_f(7);
                     f[8] = r_f(8);
                 }
-                if (EDGE) side_walls(f, g, r_f(1), r_f(3), r_g(1), r_g(3), e0, e1);
+                    if (SIDE) {
+                    float h0, h1;
+                    h0 = St::ldd(&e0, 0, float(rest_f(5)));   // the diagonals' rest values are equal
+                    h1 = St::ldd(&e1, 0, float(rest_f(5)));
+                    side_walls(f, g, r_f(1), r_f(3), r_g(1), r_g(3), h0, h1);
+                }
                 t = rawt;
                 d = da;
                 if (y < last) load(y + 1);
@@ -248,7 +231,7 @@ strip_rows(const typename Store<PREC>::S *__restrict__ src, typename Store<PREC>
                 g[0] = pair_at<PREC>(ra, 9 * 64, rest_g(0));
                 g[1] = from_left(c1, 0.f, lane);
                 g[3] = from_right(c3, 0.f, lane);
-                if (!EDGE || Y > 0) {
+                if (!ROWS || Y > 0) {
                     f[2] = pair_at<PREC>(rb, 2 * 64, rest_f(2));
                     f[5] = from_left(pair_at<PREC>(rb, 5 * 64, rest_f(5)), 0.f, lane);
                     f[6] = from_right(pair_at<PREC>(rb, 6 * 64, rest_f(6)), 0.f, lane);
@@ -259,7 +242,7 @@ strip_rows(const typename Store<PREC>::S *__restrict__ src, typename Store<PREC>
                     f[6] = pair_at<PREC>(ra, 8 * 64, rest_f(8));
                     g[2] = pair_at<PREC>(ra, 13 * 64, rest_g(4));
                 }
-                if (!EDGE || Y < ny - 1) {
+                if (!ROWS || Y < ny - 1) {
                     f[4] = pair_at<PREC>(rc, 4 * 64, rest_f(4));
                     f[7] = from_right(pair_at<PREC>(rc, 7 * 64, rest_f(7)), 0.f, lane);
                     f[8] = from_left(pair_at<PREC>(rc, 8 * 64, rest_f(8)), 0.f, lane);
@@ -270,7 +253,7 @@ strip_rows(const typename Store<PREC>::S *__restrict__ src, typename Store<PREC>
                     f[8] = pair_at<PREC>(ra, 6 * 64, rest_f(6));
                     g[4] = pair_at<PREC>(ra, 11 * 64, rest_g(2));
                 }
-                if (EDGE) {
+                if (SIDE) {
                     const int j = right_y;
                     side_walls(f, g, a1, a3, c1, c3, St::ldd(ra, (left ? 7 : 8) * 64 + j, float(rest_f(8))),
                                St::ldd(ra, (left ? 6 : 5) * 64 + j, float(rest_f(5))));
@@ -287,7 +270,7 @@ strip_rows(const typename Store<PREC>::S *__restrict__ src, typename Store<PREC>
             } else {
                 if (out) {
                     const int64_t k = (int64_t)Y * W + x;
-                    if (!EDGE || !right_x) {
+                    if (!SIDE || !right_x) {
 #pragma unroll
                         for (int i = 0; i < 9; i++) St::sdv2(dst + i * P, k, f[i], float(rest_f(i)), rng);
 #pragma unroll
@@ -313,31 +296,26 @@ strip_rows(const typename Store<PREC>::S *__restrict__ src, typename Store<PREC>
     }
 }
 
-// Unit `unit` of a grid's plan, by one warp; the edge strips' units come first.
+// Unit `unit` of a grid's plan, by one warp.
 template <int PREC, int FIELD, int TAU>
 __device__ __forceinline__ void
 strip_unit(const typename Store<PREC>::S *__restrict__ src, typename Store<PREC>::S *__restrict__ dst,
            const float *__restrict__ tsrc, float *__restrict__ tdst, const Phys<F2> &p, const StripPlan &plan, int unit,
            typename Store<PREC>::S (&ring)[3][14][64], float (&tring)[3][64])
 {
-    const int nedge = plan.edges(), ninner = plan.inner(), ny = p.ny;
-    if (unit < nedge * plan.nedge) {
-        const int j = unit % nedge, seg = unit / nedge;
-        const int ya = (int)((int64_t)ny * seg / plan.nedge), yb = (int)((int64_t)ny * (seg + 1) / plan.nedge);
-        strip_rows<PREC, FIELD, TAU, true>(src, dst, tsrc, tdst, p, j < plan.first ? j : j - plan.first + plan.end, ya, yb,
-                                           plan.lo, plan.hi, ring, tring);
-        return;
-    }
+    const int strip = unit % plan.nstrips, seg = unit / plan.nstrips, ny = p.ny;
     // the first and last segments, which hold the bottom and top wall, get 5/8
-    // of the others' rows
-    const int u = unit - nedge * plan.nedge, seg = u / ninner, strip = plan.first + u % ninner;
+    // of the others' rows: they take longer, and all units should end together
     const int total = 8 * plan.nseg - 6;
     const int ya = seg == 0 ? 0 : (int)((int64_t)ny * (8 * seg - 3) / total);
     const int yb = seg == plan.nseg - 1 ? ny : (int)((int64_t)ny * (8 * seg + 5) / total);
+    const bool side = strip < plan.first || strip >= plan.end;
     if (ya == 0 || yb == ny)
-        strip_rows<PREC, FIELD, TAU, true>(src, dst, tsrc, tdst, p, strip, ya, yb, plan.lo, plan.hi, ring, tring);
+        strip_rows<PREC, FIELD, TAU, true, true>(src, dst, tsrc, tdst, p, strip, ya, yb, plan.lo, plan.hi, ring, tring);
+    else if (side)
+        strip_rows<PREC, FIELD, TAU, true, false>(src, dst, tsrc, tdst, p, strip, ya, yb, plan.lo, plan.hi, ring, tring);
     else
-        strip_rows<PREC, FIELD, TAU, false>(src, dst, tsrc, tdst, p, strip, ya, yb, plan.lo, plan.hi, ring, tring);
+        strip_rows<PREC, FIELD, TAU, false, false>(src, dst, tsrc, tdst, p, strip, ya, yb, plan.lo, plan.hi, ring, tring);
 }
 
 }  // namespace lbm
