@@ -60,14 +60,15 @@ __device__ __forceinline__ F2 vfma(F2 a, F2 b, F2 c) { return F2(__ffma2_rn(a.v,
 // depend on the kernel that updates it: FP32 runs are compared bit for bit
 // between kernels.  So a packed kernel that takes wall nodes too says which
 // components of its pair are to be rounded as single nodes (SingleLanes), or
-// that both are (AsSingle).
+// that both are (AsSingle).  FP64 rounds the product first in nmad() and fuses
+// in pmad(): the literal law's runs keep their bits too.
 struct AsUsual {};
 struct AsSingle {};
 struct SingleLanes {
     bool x, y;
 };
 // c - a b
-__device__ __forceinline__ double nmad(double a, double b, double c, AsUsual) { return c - a * b; }
+__device__ __forceinline__ double nmad(double a, double b, double c, AsUsual) { return __dsub_rn(c, __dmul_rn(a, b)); }
 __device__ __forceinline__ float nmad(float a, float b, float c, AsUsual) { return fmaf(-a, b, c); }
 __device__ __forceinline__ F2 nmad(F2 a, F2 b, F2 c, AsUsual) { return c - a * b; }
 __device__ __forceinline__ F2 nmad(F2 a, F2 b, F2 c, SingleLanes z)
@@ -77,7 +78,7 @@ __device__ __forceinline__ F2 nmad(F2 a, F2 b, F2 c, SingleLanes z)
 }
 __device__ __forceinline__ F2 nmad(F2 a, F2 b, F2 c, AsSingle) { return vfma(-a, b, c); }
 // c + a b
-__device__ __forceinline__ double pmad(double a, double b, double c, AsUsual) { return c + a * b; }
+__device__ __forceinline__ double pmad(double a, double b, double c, AsUsual) { return fma(a, b, c); }
 __device__ __forceinline__ float pmad(float a, float b, float c, AsUsual) { return fmaf(a, b, c); }
 __device__ __forceinline__ F2 pmad(F2 a, F2 b, F2 c, AsUsual) { return c + a * b; }
 __device__ __forceinline__ F2 pmad(F2 a, F2 b, F2 c, AsSingle) { return vfma(a, b, c); }
@@ -762,8 +763,16 @@ __device__ __forceinline__ V implicit_tau(const Phys<V> &p, const V f[9], const 
         const V e_eq = vfma(rho, u2e3, V(-2) * (DEV ? r0 : rho));
         const V w = vrcp(tau);
         const V A = V(1.4 / 6.0) * (e - e_eq);
-        const V B = V(0.5) * w * nmad(rie, vfma(ux, ux, -(uy * uy)), pxx, z);
-        const V C = w * nmad(rie, ux * uy, pxy, z);
+        V pxx_neq, pxy_neq;
+        if constexpr (std::is_same<V, double>::value) {
+            pxx_neq = pxx - rie * vfma(ux, ux, -(uy * uy));
+            pxy_neq = pxy - rie * (ux * uy);
+        } else {
+            pxx_neq = nmad(rie, vfma(ux, ux, -(uy * uy)), pxx, z);
+            pxy_neq = nmad(rie, ux * uy, pxy, z);
+        }
+        const V B = V(0.5) * w * pxx_neq;
+        const V C = w * pxy_neq;
         const V bc = vfma(B, B, C * C);
         const V ss = vfma(A, A, bc);
         tau = tau_newton(p, tau, gsc * vsqrt(ss), bc, ss);
