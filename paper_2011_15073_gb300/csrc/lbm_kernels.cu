@@ -4,6 +4,7 @@
 
 #include "lbm_device.cuh"
 #include "lbm_internal.h"
+#include "lbm_nusselt.cuh"
 #include "lbm_step.cuh"
 
 namespace lbm {
@@ -139,66 +140,22 @@ __global__ void fields_kernel(const typename Store<PREC>::S *__restrict__ src,
     out[4 * n + q] = double(m.nu);
 }
 
-// FP64 block sum of one value (blockDim.x a multiple of 32, <= 1024); the
-// reduction tree is fixed, so results are reproducible run to run.
-__device__ double block_sum(double v, double *sh)
-{
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    __syncthreads();
-    if (lane == 0) sh[wid] = v;
-    __syncthreads();
-    double t = 0.0;
-    if (wid == 0) {
-        t = lane < nw ? sh[lane] : 0.0;
-        for (int o = 16; o > 0; o >>= 1) t += __shfl_down_sync(0xffffffffu, t, o);
-    }
-    return t;  // valid in thread 0
-}
-
-// Streamed temperature of node (x, y) in FP64 (thermal part of the pull).
-template <int PREC, bool REV>
-__device__ double streamed_T(const typename Store<PREC>::S *__restrict__ src,
-                             const Phys<typename Store<PREC>::R> &p, int x, int y)
-{
-    using R = typename Store<PREC>::R;
-    R f[9], g[5];
-    pull<PREC, R, REV>(src, p, x, y, f, g);
-    return (double)g[0] + (double)g[1] + (double)g[2] + (double)g[3] + (double)g[4];
-}
-
-// Wall Nusselt numbers: one block; row j of the hot wall gets
-// Nu_j = -L (9 theta_0 - theta_1 - 8) / 3, the cold wall the outward
-// L (9 theta_{nx-1} - theta_{nx-2}) / 3, theta = (T - T_c) / (T_h - T_c).
-// Rows [row_lo, row_hi) (all rows of a whole cavity, the interior rows of a
-// slab); small[0..1] the averages over them, small[6..7] the sums.
+// Wall Nusselt numbers (nusselt_rows) of rows [row_lo, row_hi) (all rows of a
+// whole cavity, the interior rows of a slab): small[0..1] the averages,
+// small[6..7] the sums.
 template <int PREC, bool REV>
 __global__ void __launch_bounds__(256)
 nusselt_kernel(const typename Store<PREC>::S *__restrict__ src, Phys<typename Store<PREC>::R> p,
                double T_hot, double T_cold, double Lw, double *__restrict__ small,
                double *__restrict__ nuloc, int row_lo, int row_hi)
 {
-    __shared__ double sh[32];
-    const double dT = T_hot - T_cold;
-    double sh_hot = 0.0, sh_cold = 0.0;
-    for (int j = row_lo + threadIdx.x; j < row_hi; j += blockDim.x) {
-        const double t0 = (streamed_T<PREC, REV>(src, p, 0, j) - T_cold) / dT;
-        const double t1 = (streamed_T<PREC, REV>(src, p, 1, j) - T_cold) / dT;
-        const double ta = (streamed_T<PREC, REV>(src, p, p.nx - 1, j) - T_cold) / dT;
-        const double tb = (streamed_T<PREC, REV>(src, p, p.nx - 2, j) - T_cold) / dT;
-        const double nh = -Lw * (9.0 * t0 - t1 - 8.0) / 3.0;
-        const double nc = Lw * (9.0 * ta - tb) / 3.0;
-        nuloc[j] = nh;
-        sh_hot += nh;
-        sh_cold += nc;
-    }
-    const double a = block_sum(sh_hot, sh);
-    const double b = block_sum(sh_cold, sh);
+    double sums[2];
+    nusselt_rows<PREC, REV>(src, p, T_hot, T_cold, Lw, nuloc, row_lo, row_hi, sums);
     if (threadIdx.x == 0) {
-        small[0] = a / (row_hi - row_lo);
-        small[1] = b / (row_hi - row_lo);
-        small[6] = a;
-        small[7] = b;
+        small[0] = sums[0] / (row_hi - row_lo);
+        small[1] = sums[1] / (row_hi - row_lo);
+        small[6] = sums[0];
+        small[7] = sums[1];
     }
 }
 
