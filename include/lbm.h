@@ -51,9 +51,11 @@ enum {
 #define LBM_TAU_ITERS_MAX 16   /* largest lbm_opts.tau_iters */
 
 /* Storage precision of the distributions.  Arithmetic is FP64 for LBM_F64
- * and FP32 otherwise.  The *D forms store the deviation of each population
- * from its rest-state value (w_i for the flow, w_i T_m for the heat): in 16
- * bits for BF16D and F16D, in 32 bits for F32D; the per-node relaxation time
+ * (a time step's collision in 64-bit fixed point, to no larger an error, under
+ * the continuous law or with n = 1) and FP32 otherwise.  The *D forms store
+ * the deviation of each population from its rest-state value (w_i for the
+ * flow, w_i T_m for the heat): in 16 bits for BF16D and F16D, in 32 bits for
+ * F32D; the per-node relaxation time
  * is then stored as FP32.  F16S and BF16S store the same 16-bit deviations
  * rounded stochastically (up or down with probability given by the distance
  * to the two neighbours; the random bits are hashed from a per-step seed

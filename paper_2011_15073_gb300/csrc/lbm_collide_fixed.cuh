@@ -162,16 +162,15 @@ inline Q<N> q_host(double x, int &ok)
         ok = 0;
         return Q<N>{0};
     }
-    return Q<N>{llrintl(ldexpl((long double)x, N))};
+    return q_of<N>(x);
 }
 inline Q<57> log2_host(double x, double least, int &ok)
 {
-    const long double l = log2l((long double)x);
-    if (!(l >= least && l < 32.0L)) {
+    if (!(x >= least && x < 0x1p32)) {
         ok = 0;
         return Q<57>{0};
     }
-    return Q<57>{llrintl(ldexpl(l, 57))};
+    return Q<57>{((int64_t)((int)(bits_of(x) >> 52) - 1023) << 57) + log2_mantissa_q57(bits_of(x))};
 }
 inline FixedParams fixed_params(double eps, double gbeta, double omegaT, double s_e, double s_p, double n,
                                 double gamma_scale, double gamma1, double gamma2, int clamp_mode)
@@ -184,9 +183,9 @@ inline FixedParams fixed_params(double eps, double gbeta, double omegaT, double 
     f.s_e3 = q_host<62>(s_e / 3.0, f.ok);
     f.inv_eps = q_host<60>(1.0 / eps, f.ok);
     f.nm1 = q_host<62>(n - 1.0, f.ok);
-    f.log_scale = log2_host(1.5 * gamma_scale, 0.0, f.ok);
-    f.log_g1 = log2_host(gamma1, -32.0, f.ok);
-    f.log_g2 = log2_host(gamma2, -32.0, f.ok);
+    f.log_scale = log2_host(1.5 * gamma_scale, 1.0, f.ok);
+    f.log_g1 = log2_host(gamma1, 0x1p-31, f.ok);
+    f.log_g2 = log2_host(gamma2, 0x1p-31, f.ok);
     return f;
 }
 
