@@ -85,6 +85,19 @@ def step_kernel_name(prec, layout, tau_iters, staging, N):
 
 def bytes_per_node(prec, tau_iters=0):
     return BYTES_PER_NODE[prec] - (TAU_BYTES[prec] if tau_iters else 0)
+
+
+def steps_per_launch(prec, layout, tau_iters, staging, N):
+    """Time steps one launch of lbm_step takes on a large N x N cavity: two with
+    FP32 storage in the two-buffer layout from 600,000 nodes on (2,000,000 with
+    the implicit tau), the rule of lbm_strip.cu."""
+    return 2 if prec in ("f32", "f32d") and not layout and not staging and N * N >= (2000000 if tau_iters else 600000) else 1
+
+
+def launch_label(prec, layout, tau_iters, staging, N):
+    if steps_per_launch(prec, layout, tau_iters, staging, N) == 2:
+        return "strip_kernel (two steps per launch)"
+    return step_kernel_name(prec, layout, tau_iters, staging, N)
 CASE = dict(n=0.6, Da=1e-3, Ra=1e5, Pr=6.2, porosity=0.6)
 FALLBACK_HBM_GBS = 6800.0
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "traffic.txt")
@@ -97,7 +110,8 @@ PRECISION_FILE = os.path.join(ROOT, "profiles", "precision_study_512.txt")
 # and staged kernels are not among them.
 # the files that define the step kernels' arithmetic and which kernel runs
 # (host-only files are left out: they do not change a measured figure)
-RECORD_SOURCES = ("lbm_device.cuh", "lbm_round.cuh", "lbm_step.cuh", "lbm_kernels.cu")
+RECORD_SOURCES = ("lbm_device.cuh", "lbm_round.cuh", "lbm_step.cuh", "lbm_kernels.cu", "lbm_strip.cuh", "lbm_strip.cu",
+                  "lbm_fixed.cuh", "lbm_collide_fixed.cuh")
 
 
 def kernel_source_hash():
@@ -374,7 +388,8 @@ def time_ours(lbm, torch, N, prec, steps, warmup, delta, stream, layout=0, tau_i
         torch.cuda.synchronize()
         total = t0.elapsed_time(t1) / 1e3
         kern = sum(a.elapsed_time(b) for a, b in ev) / 1e3 / (steps * delta)
-        launches = steps * (delta + 1 + 2)
+        spl = steps_per_launch(prec, layout, tau_iters, staging, N)
+        launches = steps * (delta // spl + delta % spl + 1 + 2)
         return total, kern, launches, nu
     finally:
         cav.close()
@@ -1051,7 +1066,9 @@ def main():
     units = whole_job_units(world, N, delta, args.steps)
     mlups = units / total / 1e6
     peak, peak_src = hbm_peak()
-    bpn_main = bytes_per_node(prec, args.tau_iters)
+    # HBM bytes per node update: a launch of two steps reads and writes the state once for both
+    spl = steps_per_launch(prec, args.layout, args.tau_iters, args.staging, N)
+    bpn_main = bytes_per_node(prec, args.tau_iters) / spl
     achieved = bpn_main * N * N / kern / 1e9
     key_main = prec + (f"@tau{args.tau_iters}" if args.tau_iters else "") + \
         {0: "", 1: "@reg", 3: "@quad"}[args.staging] + ("@aa" if args.layout else "")
@@ -1061,7 +1078,7 @@ def main():
         vs, vd = 2, args.variant_delta
         vp, vl, vt, vg = parse_variant(v)
         tv, kv, _, nuv = time_ours(lbm, torch, N, vp, vs, 1, vd, stream, layout=vl, tau_iters=vt, staging=vg)
-        bpn = bytes_per_node(vp, vt)
+        bpn = bytes_per_node(vp, vt) / steps_per_launch(vp, vl, vt, vg, N)
         av = bpn * N * N / kv / 1e9
         variants[v] = {"MLUPS": N * N * vd * vs / tv / 1e6, "kernel_MLUPS": N * N / kv / 1e6,
                        "fused_steps_per_bench_step": vd,
@@ -1070,7 +1087,7 @@ def main():
                        "tau": f"implicit, {vt} Newton steps" if vt else "lagged (stored)",
                        "dnu_rel_vs_f64_512": recorded_dnu(vp),
                        "staging": staging_label(vp, vl, vt, vg, N),
-                       "kernel": step_kernel_name(vp, vl, vt, vg, N),
+                       "kernel": launch_label(vp, vl, vt, vg, N),
                        "nu_hot": nuv}
         if v == "f64":
             ipn = recorded("f64_fp64_inst_per_node")
@@ -1111,9 +1128,8 @@ def main():
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
                      "frac": achieved / peak, "traffic": recorded_traffic(key_main, N),
                      "peak_source": peak_src,
-                     "kernel": step_kernel_name(prec, args.layout, args.tau_iters, args.staging, N) +
-                               f"<{key_main}>",
-                     "bytes_per_node": bpn_main, "avg_launch_us": kern * 1e6,
+                     "kernel": launch_label(prec, args.layout, args.tau_iters, args.staging, N) + f"<{key_main}>",
+                     "bytes_per_node": bpn_main, "steps_per_launch": spl, "avg_launch_us": kern * spl * 1e6,
                      # the arithmetic side of the same kernel: FMA-pipe activity (ncu, 2048^2)
                      "fma_pipe_active": recorded(key_main + "_fma_pipe_active")},
         "cpu_baseline": cpu,
