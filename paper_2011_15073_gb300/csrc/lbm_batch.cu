@@ -484,6 +484,10 @@ cudaError_t launch_batch_step(lbm_batch *b, StepAt at)
 // Whether lbm_batch_step takes two steps per launch: FP32 storage without a
 // per-node Darcy field, and enough nodes to fill the chip (as two_steps() for
 // one cavity; the smallest widths share a lane between both side walls).
+// Widths that fill little of their strips gain too (1.5 M nodes, FP32
+// deviations, us per step, tuned tiles / strips): 64 x 64 73 / 44, 64 x 400
+// 67 / 37, 90 x 90 62 / 35, 118 x 118 52 / 25, 128 x 128 46 / 33, 300 x 300
+// 45 / 22; at 0.7 M nodes 32 / 22, 31 / 19, 25 / 16, 23 / 14, 21 / 16, 19 / 12.
 bool batch_strips(const lbm_batch *b)
 {
     if (b->any_field || (b->opts.prec != LBM_F32 && b->opts.prec != LBM_F32D) || b->opts.staging != 0) return false;
