@@ -482,12 +482,16 @@ cudaError_t launch_batch_step(lbm_batch *b, StepAt at)
 }
 
 // Whether lbm_batch_step takes two steps per launch: FP32 storage without a
-// per-node Darcy field, and enough nodes to fill the chip (as two_steps() for
-// one cavity; the smallest widths share a lane between both side walls).
+// per-node Darcy field, and enough nodes to fill the chip (the smallest
+// widths share a lane between both side walls).
 // Widths that fill little of their strips gain too (1.5 M nodes, FP32
 // deviations, us per step, tuned tiles / strips): 64 x 64 73 / 44, 64 x 400
 // 67 / 37, 90 x 90 62 / 35, 118 x 118 52 / 25, 128 x 128 46 / 33, 300 x 300
 // 45 / 22; at 0.7 M nodes 32 / 22, 31 / 19, 25 / 16, 23 / 14, 21 / 16, 19 / 12.
+// The line: at 0.45 M nodes 64 x 64 21.2 / 15.1, 128 x 128 12.7 / 11.6,
+// 256 x 256 10.5 / 10.4; at 0.24 M 12.8 / 10.7, 9.2 / 9.5, 7.9 / 7.4.  With the
+// implicit tau (as two_steps() for one cavity) 29 / 24, 16.8 / 20.6, 14 / 16.7
+// at 0.45 M.
 bool batch_strips(const lbm_batch *b)
 {
     if (b->any_field || (b->opts.prec != LBM_F32 && b->opts.prec != LBM_F32D) || b->opts.staging != 0) return false;
@@ -496,7 +500,7 @@ bool batch_strips(const lbm_batch *b)
         if (c->nx < 64 || c->ny < 16) return false;
         nodes += (int64_t)c->nx * c->ny;
     }
-    return nodes >= (b->opts.tau_iters > 0 ? 2000000 : 600000);
+    return nodes >= (b->opts.tau_iters > 0 ? 2000000 : 300000);
 }
 
 cudaError_t launch_batch_strips(lbm_batch *b, int odd)
