@@ -20,8 +20,10 @@
 // most 2^-60 or so, without bias, and the results are rounded to FP64 once; FP64 arithmetic
 // rounds every one of those operations, to 2^-53 of populations between 0.02
 // and 0.5.  What a node holds outside the ranges below (populations outside
-// (2^-15, 1), |j| >= 1/4, a density outside (1/2, 2), ..., NaN) is left to the
-// plain FP64 collision: collide_fixed() returns false.
+// (2^-15, 1), |j| >= 1/4, a density outside (1/2, 3/2), ..., NaN) is left to the
+// plain FP64 collision: collide_fixed() returns false.  The ranges are those in
+// which no intermediate leaves its format; a bound stands at each test and each
+// sum that needs one.
 //
 // Q<N> holds a value times 2^N in 64 bits.
 #pragma once
@@ -56,9 +58,11 @@ __host__ __device__ __forceinline__ Q<M> as(Q<N> a)
         return Q<M>{(a.v + (1ll << (N - M - 1))) >> (N - M)};
 }
 
-// High 64 bits of a signed product, |a|, |b| <= 2^62, to within 3/4, without
+// High 64 bits of a signed product, |a|, |b| < 2^63 - 2^32, to within 3/4, without
 // bias.  Low words are taken as signed and the high words corrected for it,
 // so that all three products are signed ones; the low-low product is dropped.
+// (The corrected high words are then below 2^31, and s below
+// 2 (2^31 - 1) 2^31 + 2^31 < 2^63.)
 __host__ __device__ __forceinline__ int64_t smulhi(int64_t a, int64_t b)
 {
     const int32_t al = (int32_t)a, bl = (int32_t)b;
@@ -236,10 +240,10 @@ __host__ __device__ __forceinline__ Q<61> rcp_density(Q<60> r)
 __host__ __device__ __forceinline__ bool collide_fixed(const FixedParams &p, double nu3, bool quadratic_drag, double heK, double eK, double c1,
                                                        double eFsK, double f[9], double g[5], double &tau)
 {
-    // ranges of the inputs: populations in [2^-15, 1), |g| < 1, tau in [1/4, 2^10)
+    // ranges of the inputs: populations in [2^-15, 1), |g_0| < 1/2, |g_i| < 1, tau in [1/4, 2^10)
     uint32_t bad = 0;
     for (int i = 0; i < 9; i++) bad |= (uint32_t)(hi_word(f[i]) - 0x3f000000u >= 0x00f00000u);
-    for (int i = 0; i < 5; i++) bad |= (uint32_t)((hi_word(g[i]) & 0x7fffffffu) >= 0x3ff00000u);
+    for (int i = 0; i < 5; i++) bad |= (uint32_t)((hi_word(g[i]) & 0x7fffffffu) >= (i == 0 ? 0x3fe00000u : 0x3ff00000u));
     bad |= (uint32_t)(hi_word(tau) - 0x3fd00000u >= 0x00c00000u);
     if (bad) return false;
 
@@ -262,10 +266,15 @@ __host__ __device__ __forceinline__ bool collide_fixed(const FixedParams &p, dou
     const Q<60> t0 = G[0] + s14 - (one >> 1);   // T - T_m
     const Q<60> n1 = G[1] - G[3], n2 = G[2] - G[4], n4 = g13 - g24;
     const Q<60> n3 = s14 - (G[0] << 2) + Q<60>{384307168202282325}, n3n = 3 * n3 + (t0 << 1);   // without its rest value -1/3
-    // density in (1/2, 2), |j| < 1/4, |T - T_m| < 1, ...
-    bad |= (uint32_t)((uint64_t)rho.v - (1ull << 59) >= (3ull << 59));
-    bad |= outside<58>(jx) | outside<58>(jy) | outside<60>(t0) | outside<59>(n1) | outside<59>(n2) | outside<59>(n4) |
-           outside<60>(n3n);
+    // density in (1/2, 3/2), |j| < 1/4, |T - T_m| < 1, ...  r0, the momenta and t0
+    // lie within +-8 whatever the populations, so that what is tested has not
+    // wrapped.  n3n = 5 t0 + 5/2 - 15 g_0 has: but with |t0| < 1 and |g_0| < 1/2 it is
+    // in (-10, 15), and what wraps (by 16) misses (-1, 1).  In the same way
+    // 7 r0 + e, in (-6, 17/2), misses (-2, 2) and 7 r0 - 2 ep, in (-21/2, 23/2),
+    // (-4, 4): these two bound the numerators of a1 and a2, and are tested here,
+    // where few values are held (f and g stay until the last refusal).
+    bad |= outside<59>(r0) | outside<58>(jx) | outside<58>(jy) | outside<60>(t0) | outside<59>(n1) | outside<59>(n2) |
+           outside<59>(n4) | outside<60>(n3n) | outside<61>(7 * r0 + e) | outside<62>(7 * r0 - (ep << 1));
     if (bad) return false;
 
     // velocity v and the porous solve u = v / (c0 + sqrt(c0^2 + c1 |v|)), the latter in FP64
@@ -292,13 +301,17 @@ __host__ __device__ __forceinline__ bool collide_fixed(const FixedParams &p, dou
     const Q<62> drq = q_of<62>(drag);
     const Q<64> ux = as<64>(as<64>(vx) * idq), uy = as<64>(as<64>(vy) * idq);
     const Q<62> fx = drq * ux, fy = drq * uy + buoy;
-    // equilibria: rho u u / eps
+    // equilibria: rho u u / eps; |u| <= |v| < 1/4 each way and rho / eps < 6, so K3 < 9/4
     const Q<60> rie = as<60>(as<61>(rho) * p.inv_eps);
     const Q<64> xx = ux * ux, yy = uy * uy, xy = ux * uy;
     const Q<60> Kxx = (xx - yy) * rie, Kxy = xy * rie, K3 = 3 * ((xx + yy) * rie);
     const Q<60> e_eq = K3 - (r0 << 1), ep_eq = r0 - K3;
     const Q<60> en = e - e_eq, pn = pxx - Kxx, cn = pxy - Kxy;
-    if (outside<60>(fx) | outside<60>(fy) | outside<57>(pn) | outside<57>(cn)) return false;
+    // K3 < 1/4; |F| < 1/16, so that the forcing's products with u and rho / eps stay
+    // below 3/16 (Fxx: 3/8).  Then the numerators of a1 and a2 are below
+    // 4 + 7/4 + 27/16 (the format holds 8), pn + Fxx / 2 and cn + Fxy / 2 below 5/16
+    // (Q64 holds 1/2).
+    if (outside<58>(fx) | outside<58>(fy) | outside<57>(pn) | outside<57>(cn) | outside<58>(K3)) return false;
     const Q<64> Fx = as<64>(fx), Fy = as<64>(fy);
     double D = 1.0;
     if (p.nm1.v != 0) {
@@ -330,6 +343,7 @@ __host__ __device__ __forceinline__ bool collide_fixed(const FixedParams &p, dou
     const Q<60> a1 = (7 * e_eq - (e << 1) + 9 * R) * n180;
     const Q<60> a2 = (7 * ep_eq - (ep << 1) - 9 * R) * n180;
     const Q<60> a3 = (rux + (rFx >> 1)) * n6, a5 = (ruy + (rFy >> 1)) * n6;
+    // |qx| = |jx - 3 (f1 - f3)| < 13/4, the sum below 6
     const Q<60> a4 = Q<60>{0} - (qx + 6 * rux + (rFx << 1)) * n60, a6 = Q<60>{0} - (qy + 6 * ruy + (rFy << 1)) * n60;
     const Q<60> a7 = (pxx + Fxx - as<60>(as<64>(pn + (Fxx >> 1)) * wq)) >> 2;
     const Q<60> a8 = (pxy + Fxy - as<60>(as<64>(cn + (Fxy >> 1)) * wq)) >> 2;
