@@ -245,6 +245,15 @@ __host__ __device__ __forceinline__ bool collide_fixed(const FixedParams &p, dou
     for (int i = 0; i < 9; i++) bad |= (uint32_t)(hi_word(f[i]) - 0x3f000000u >= 0x00f00000u);
     for (int i = 0; i < 5; i++) bad |= (uint32_t)((hi_word(g[i]) & 0x7fffffffu) >= (i == 0 ? 0x3fe00000u : 0x3ff00000u));
     bad |= (uint32_t)(hi_word(tau) - 0x3fd00000u >= 0x00c00000u);
+    // the Darcy drag below 1, coefficients for which 2^-64 in |v|^2 is below FP64's own
+    // rounding.  Before any other work: on a small grid a small Darcy number takes every node
+    // beyond this, and the FP64 collision then comes on top (512^2, Da = 1e-7, n = 0.8: 166.2 us per
+    // step as with FP64 alone; with the test after the velocity solve 176.4; drags on both sides of 1
+    // in one warp, Da = 1e-6: 172).
+    const double nu_prev = fma(tau, 1.0 / 3.0, -1.0 / 6.0);
+    double drag = -eK * nu_prev;
+    bad |= (uint32_t)((hi_word(drag) & 0x7fffffffu) >= 0x3ff00000u) | (uint32_t)(hi_word(c1) >= 0x40100000u) |
+           (uint32_t)(hi_word(eFsK) >= 0x40200000u);
     if (bad) return false;
 
     Q<60> F[9], G[5];
@@ -282,9 +291,8 @@ __host__ __device__ __forceinline__ bool collide_fixed(const FixedParams &p, dou
     const Q<62> buoy = as<62>(t0) * p.buoy;   // eps g beta (T - T_m)
     const Q<62> vx = as<62>(as<64>(jx) * irho), vy = as<62>(as<64>(jy) * irho) + (buoy >> 1);
     if (outside<60>(vx) | outside<60>(vy)) return false;
-    const double nu_prev = fma(tau, 1.0 / 3.0, -1.0 / 6.0);
     const double c0 = fma(heK, nu_prev, 0.5);
-    double iden, drag = -eK * nu_prev;
+    double iden;
     if (quadratic_drag) {
         const Q<64> wx = as<64>(vx), wy = as<64>(vy);
         const double vmag = sqrt_or_ieee(double_of(wx * wx + wy * wy));
@@ -293,9 +301,8 @@ __host__ __device__ __forceinline__ bool collide_fixed(const FixedParams &p, dou
     } else {
         iden = rcp_or_ieee(c0 + c0);
     }
-    // 1 / den in (0, 1], |drag| < 1, coefficients for which 2^-64 in |v|^2 is below FP64's own rounding
+    // 1 / den in (0, 1], |drag| < 1
     bad |= (uint32_t)(hi_word(iden) > 0x3ff00000u) | (uint32_t)((hi_word(drag) & 0x7fffffffu) >= 0x3ff00000u);
-    bad |= (uint32_t)(hi_word(c1) >= 0x40100000u) | (uint32_t)(hi_word(eFsK) >= 0x40200000u);
     if (bad) return false;
     const Q<62> idq = q_of<62>(iden);
     const Q<62> drq = q_of<62>(drag);
