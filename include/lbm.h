@@ -323,9 +323,11 @@ void lbm_batch_destroy(lbm_batch *batch);
 /* Borrow case i's context for state I/O, fields or Nu (do not destroy it). */
 int lbm_batch_get_case(lbm_batch *batch, int i, lbm_ctx **ctx);
 
-/* Advance every case k steps (one launch per step of the plan below, or with
- * FP32 storage and many nodes per two steps; the values are the same).
- * Asynchronous. */
+/* Advance every case k steps.  With FP32 storage, no Darcy field and many nodes
+ * (300,000, or 2,000,000 with the implicit tau, in grids of 64 columns and 16
+ * rows or more) one launch takes two steps, unless lbm_batch_set_plan has set a
+ * plan; what is left of that, and every other batch, runs on the plan below.
+ * The values are the same.  Asynchronous. */
 int lbm_batch_step(lbm_batch *batch, int64_t k);
 
 /* Run every case until its residual (as lbm_run_to_steady) falls below tol,
@@ -363,11 +365,14 @@ int lbm_batch_nusselt(lbm_batch *batch, double *nu_hot, double *nu_cold);
 enum { LBM_BATCH_PER_STEP = 0, LBM_BATCH_PERSISTENT = 1 };
 
 /* Set the plan: mode as above, threads 64, 128 or 256 (tile = 2 x threads
- * nodes, or threads nodes in FP64), blocks_per_sm 1..64.  Errors:
+ * nodes, or threads nodes in FP64), blocks_per_sm 1..64.  lbm_batch_step then
+ * takes every step on it, until lbm_batch_tune chooses another.  Errors:
  * LBM_ERR_ARG, LBM_ERR_UNSUPPORTED (no block of the persistent kernel fits
  * on an SM), LBM_ERR_CUDA. */
 int lbm_batch_set_plan(lbm_batch *batch, int mode, int threads, int blocks_per_sm);
-/* Read the plan in effect (blocks_per_sm after the residency cap). */
+/* Read the plan in effect (blocks_per_sm after the residency cap): the one that
+ * lbm_batch_run_to_steady runs on, and lbm_batch_step but for the two-step
+ * launches described there. */
 int lbm_batch_get_plan(const lbm_batch *batch, int *mode, int *threads, int *blocks_per_sm);
 /* Clock cycles a persistent block waits at a barrier before it gives up
  * (default 2^31, about one second); cycles >= 1. */
@@ -377,7 +382,9 @@ int lbm_batch_set_wait_budget(lbm_batch *batch, int64_t cycles);
  * (64, 128, 256) x blocks per SM (2, 4, 8, 16, 32; persistent: those that
  * fit) on copies of the current states (restored afterwards) and keep the
  * fastest; *threads_out (may be NULL) receives its block size and
- * lbm_batch_get_plan the rest. */
+ * lbm_batch_get_plan the rest.  The two-step launches of lbm_batch_step have no
+ * such choices and are not among them; they stay in use (again, after
+ * lbm_batch_set_plan) where lbm_batch_step takes them. */
 int lbm_batch_tune(lbm_batch *batch, int steps, int *threads_out);
 
 /* ------------------------------------------------- row-slab decomposition

@@ -346,6 +346,7 @@ struct lbm_batch {
     int threads = 128;
     int blocks_per_sm = 8;
     int mode = LBM_BATCH_PER_STEP;
+    bool plan_set = false;   // by lbm_batch_set_plan: lbm_batch_step keeps to it
     long long budget = 1ll << 31;   // clock cycles a persistent block waits at a barrier
     int ntiles = 0;
     bool any_field = false;   // some case has a per-node Darcy field
@@ -482,8 +483,9 @@ cudaError_t launch_batch_step(lbm_batch *b, StepAt at)
 }
 
 // Whether lbm_batch_step takes two steps per launch: FP32 storage without a
-// per-node Darcy field, and enough nodes to fill the chip (the smallest
-// widths share a lane between both side walls).
+// per-node Darcy field, enough nodes to fill the chip (the smallest widths
+// share a lane between both side walls), and no plan set by the caller, who may
+// count on its launches, its barrier's budget and its errors.
 // Widths that fill little of their strips gain too (1.5 M nodes, FP32
 // deviations, us per step, tuned tiles / strips): 64 x 64 73 / 44, 64 x 400
 // 67 / 37, 90 x 90 62 / 35, 118 x 118 52 / 25, 128 x 128 46 / 33, 300 x 300
@@ -494,7 +496,7 @@ cudaError_t launch_batch_step(lbm_batch *b, StepAt at)
 // at 0.45 M.
 bool batch_strips(const lbm_batch *b)
 {
-    if (b->any_field || (b->opts.prec != LBM_F32 && b->opts.prec != LBM_F32D) || b->opts.staging != 0) return false;
+    if (b->plan_set || b->any_field || (b->opts.prec != LBM_F32 && b->opts.prec != LBM_F32D) || b->opts.staging != 0) return false;
     int64_t nodes = 0;
     for (const lbm_ctx *c : b->sub) {
         if (c->nx < 64 || c->ny < 16) return false;
@@ -895,6 +897,7 @@ int lbm_batch_set_plan(lbm_batch *b, int mode, int threads, int blocks_per_sm)
         return LBM_ERR_UNSUPPORTED;
     }
     b->blocks_per_sm = blocks_per_sm;
+    b->plan_set = true;
     return upload_cases(b);
 }
 
@@ -1005,6 +1008,7 @@ int lbm_batch_tune(lbm_batch *b, int steps, int *threads_out)
     b->mode = best.mode;
     b->threads = best.threads;
     b->blocks_per_sm = best.bps;
+    b->plan_set = false;
     if (rc == LBM_OK) rc = upload_cases(b);
     if (rc == LBM_OK) rc = batch_err(b);
     if (threads_out) *threads_out = best.threads;

@@ -425,12 +425,13 @@ class Batch:
         return hot, cold
 
     def tune(self, steps=200):
+        """Choose the plan by timing; step() may take two-step launches beside it (lbm.h)."""
         t = ctypes.c_int()
         _check(lib().lbm_batch_tune(self.h, int(steps), ctypes.byref(t)), "lbm_batch_tune")
         return t.value
 
     def set_plan(self, mode, threads=128, blocks_per_sm=8):
-        """mode 'per_step' / 'persistent' (or 0 / 1)."""
+        """mode 'per_step' / 'persistent' (or 0 / 1); step() keeps to it until the next tune()."""
         m = {"per_step": 0, "persistent": 1}.get(mode, mode)
         _check(lib().lbm_batch_set_plan(self.h, int(m), int(threads), int(blocks_per_sm)), "lbm_batch_set_plan")
 
