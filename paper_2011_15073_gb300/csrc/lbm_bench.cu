@@ -1,10 +1,11 @@
-// lbm_bench.cu -- FMA-throughput probes (include/lbm_bench.h): the measured
-// ALU peaks that the FP64 step kernel's roofline and the FMA-pipe activity of
-// the FP32 kernels are compared with.
+// lbm_bench.cu -- measurement helpers (include/lbm_bench.h): FMA-throughput
+// probes, the measured ALU peaks that the FP64 step kernel's roofline and the
+// FMA-pipe activity of the FP32 kernels are compared with, and the rule by
+// which lbm_step takes several steps per launch.
 #include <cuda_runtime.h>
 
-#include "lbm.h"
 #include "lbm_bench.h"
+#include "lbm_internal.h"
 
 namespace {
 
@@ -89,4 +90,22 @@ extern "C" int lbm_bench_fma_peak(int kind, int device, int reps, double *fma_pe
     if (e1) cudaEventDestroy(e1);
     cudaFree(out);
     return rc;
+}
+
+extern "C" int lbm_bench_steps_per_launch(int nx, int ny, const lbm_opts *opts, int sms, int *steps, int *kernel)
+{
+    if (!opts || !steps || nx < 2 || ny < 2 || sms < 0) return LBM_ERR_ARG;
+    if (sms == 0) {
+        int dev = opts->device;
+        if ((dev < 0 && cudaGetDevice(&dev) != cudaSuccess) ||
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+            cudaGetLastError();
+            return LBM_ERR_CUDA;
+        }
+    }
+    const bool strips = lbm::two_steps(nx, ny, *opts);
+    const int tile = lbm::tile_steps(nx, ny, *opts, sms);
+    *steps = strips ? 2 : (tile > 1 ? tile : 1);
+    if (kernel) *kernel = strips ? LBM_LAUNCH_STRIPS : (tile > 1 ? LBM_LAUNCH_TILE : LBM_LAUNCH_STEP);
+    return LBM_OK;
 }

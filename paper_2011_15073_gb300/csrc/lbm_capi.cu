@@ -54,14 +54,15 @@ int graph_parity(const lbm_ctx *c) { return c->opts.layout == 1 ? (c->aa_form_o 
 // Steps that one launch takes where several are due (1: one).
 int steps_per_launch(const lbm_ctx *c)
 {
-    if (lbm::two_steps(c)) return 2;
-    const int m = lbm::tile_steps(c);
+    if (lbm::two_steps(c->nx, c->ny, c->opts)) return 2;
+    const int m = lbm::tile_steps(c->nx, c->ny, c->opts, c->sms);
     return m > 1 ? m : 1;
 }
 // m = 1, or a number of steps up to steps_per_launch() that a launch can take
 cudaError_t launch_steps(lbm_ctx *c, int m)
 {
-    return m == 1 ? lbm::launch_step(c) : (lbm::two_steps(c) ? lbm::launch_two_steps(c) : lbm::launch_tile(c, m));
+    if (m == 1) return lbm::launch_step(c);
+    return lbm::two_steps(c->nx, c->ny, c->opts) ? lbm::launch_two_steps(c) : lbm::launch_tile(c, m);
 }
 
 // Capture G step launches on the context's stream into an executable graph
@@ -260,6 +261,7 @@ int init_ctx(lbm_ctx *c)
     } else {
         CK(cudaGetDevice(&c->device));
     }
+    CK(cudaDeviceGetAttribute(&c->sms, cudaDevAttrMultiProcessorCount, c->device));
     const size_t es = store_elem(c->opts.prec), ts = tau_elem(c->opts.prec);
     c->pitch = ((int64_t)c->nx + 63) / 64 * 64;
     c->plane = c->pitch * c->ny;

@@ -33,6 +33,7 @@ struct Launch {
 struct lbm_ctx {
     int nx = 0, ny = 0;
     int device = 0;
+    int sms = 0;                   // SMs of that device
     lbm_opts opts{};
     lbm_lattice lat{};
     int64_t pitch = 0, plane = 0;  // elements
@@ -78,9 +79,9 @@ cudaError_t launch_step(lbm_ctx *c);
 // Several steps in one launch, the same values as launch_step calls bit for
 // bit: two on large grids (lbm_strip.cu) where two_steps() says that it pays,
 // two or four on small ones (lbm_tile.cu) where tile_steps() does (0: not).
-bool two_steps(const lbm_ctx *c);
+bool two_steps(int nx, int ny, const lbm_opts &o);
 cudaError_t launch_two_steps(lbm_ctx *c);
-int tile_steps(const lbm_ctx *c);
+int tile_steps(int nx, int ny, const lbm_opts &o, int sms);
 cudaError_t launch_tile(lbm_ctx *c, int steps);
 // Write the context's step count to d_step_base (before a step-graph replay).
 cudaError_t launch_set_step_base(lbm_ctx *c);

@@ -302,9 +302,9 @@ static cudaError_t init_t(lbm_ctx *c)
 // which has its own FP64 pipe (160^2: 128 threads 9.1 us in fixed point and
 // 36.1 us in FP64 arithmetic, 64 threads 7.1 and 24.7, 32 threads 6.8 and
 // 19.2; 1000 x 1100: the same for all).  A grid with no more warps than the
-// 608 partitions of the chip has nothing to spread, and starts faster in
-// blocks of two (64^2: 4.6 against 4.9 us).
-static int f64_block(const lbm_ctx *c) { return (int64_t)((c->nx + 31) / 32) * c->ny <= 608 ? 64 : 32; }
+// chip has partitions (four per SM) has nothing to spread, and starts faster
+// in blocks of two (64^2: 4.6 against 4.9 us).
+static int f64_block(const lbm_ctx *c) { return (int64_t)((c->nx + 31) / 32) * c->ny <= 4 * c->sms ? 64 : 32; }
 
 template <int PREC, int TAU>
 static cudaError_t step_buffers_tau(lbm_ctx *c, const void *src, void *dst, const void *tsrc, void *tdst)

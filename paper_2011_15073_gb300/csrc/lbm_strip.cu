@@ -25,7 +25,7 @@ cudaError_t strip_tau(lbm_ctx *c)
     const int s = c->cur, d = 1 - s;
     // as many units as warps fit on the chip at once (twice as many with the
     // implicit tau)
-    const int slots = 152 * strip_blocks<TAU>() * (TAU == 1 ? 2 : 1);
+    const int slots = c->sms * strip_blocks<TAU>() * (TAU == 1 ? 2 : 1);
     StripPlan plan = strip_plan(c->nx);
     plan.cut(c->ny, slots / plan.nstrips);
     const int blocks = plan.units();
@@ -50,11 +50,11 @@ cudaError_t strip_t(lbm_ctx *c)
 // a segment of four rows takes six rows' first steps, one after the other.
 // The 16-bit storages are bound by instruction issue, not by HBM, and keep
 // their four-node kernel.
-bool two_steps(const lbm_ctx *c)
+bool two_steps(int nx, int ny, const lbm_opts &o)
 {
-    if (c->opts.layout != 0 || c->opts.staging != 0 || c->nx < 128 || c->ny < 64) return false;
-    if (c->opts.prec != LBM_F32 && c->opts.prec != LBM_F32D) return false;
-    return (int64_t)c->nx * c->ny >= (c->opts.tau_iters > 0 ? 2000000 : 600000);
+    if (o.layout != 0 || o.staging != 0 || nx < 128 || ny < 64) return false;
+    if (o.prec != LBM_F32 && o.prec != LBM_F32D) return false;
+    return (int64_t)nx * ny >= (o.tau_iters > 0 ? 2000000 : 600000);
 }
 
 cudaError_t launch_two_steps(lbm_ctx *c)

@@ -207,10 +207,10 @@ tile_kernel(const typename Store<PREC>::S *__restrict__ src, typename Store<PREC
     }
 }
 
-dim3 tile_grid(const lbm_ctx *c, int steps)
+dim3 tile_grid(int nx, int ny, int steps)
 {
     const int cols = 64 - 2 * steps, rows = kTileRows - 2 * (steps - 1);
-    return dim3((c->nx + cols - 1) / cols, (c->ny + rows - 1) / rows);
+    return dim3((nx + cols - 1) / cols, (ny + rows - 1) / rows);
 }
 
 template <int PREC, int TAU>
@@ -218,7 +218,7 @@ cudaError_t tile_tau(lbm_ctx *c, int steps)
 {
     using S = typename Store<PREC>::S;
     const int s = c->cur, d = 1 - s;
-    const dim3 grid = tile_grid(c, steps);
+    const dim3 grid = tile_grid(c->nx, c->ny, steps);
     auto *kern = c->d_da ? tile_kernel<PREC, 1, TAU> : tile_kernel<PREC, 0, TAU>;
     const int smem = 4 * kTileRows * 4 * 32 * (int)sizeof(float2);
     if (const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem)) return e;
@@ -236,16 +236,16 @@ cudaError_t tile_t(lbm_ctx *c, int steps)
 
 }  // namespace
 
-// As many steps as leave one block per SM: a second wave of blocks costs more
+// As many steps as leave one block on each of the `sms` SMs: a second wave of blocks costs more
 // than the launches saved (384^2: 3.4 us a step in two waves of four steps, 3.7
 // one by one; 512^2: 6.4 and 4.9).
-int tile_steps(const lbm_ctx *c)
+int tile_steps(int nx, int ny, const lbm_opts &o, int sms)
 {
-    if (c->opts.layout != 0 || c->opts.staging != 0 || c->nx < 64) return 0;
-    if (c->opts.prec != LBM_F32 && c->opts.prec != LBM_F32D) return 0;
+    if (o.layout != 0 || o.staging != 0 || nx < 64) return 0;
+    if (o.prec != LBM_F32 && o.prec != LBM_F32D) return 0;
     for (int steps : {4, 2}) {
-        const dim3 g = tile_grid(c, steps);
-        if ((int64_t)g.x * g.y <= 152) return steps;
+        const dim3 g = tile_grid(nx, ny, steps);
+        if ((int64_t)g.x * g.y <= sms) return steps;
     }
     return 0;
 }

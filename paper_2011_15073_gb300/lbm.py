@@ -113,6 +113,8 @@ SIGNATURES = [
     ("lbm_debug_padding_canary", ctypes.c_int, [_VP, ctypes.POINTER(ctypes.c_ulonglong)]),
     ("lbm_debug_sr_pairs", ctypes.c_int, [ctypes.c_int, ctypes.c_int, _VP, _VP, _VP, ctypes.c_size_t]),
     ("lbm_bench_fma_peak", ctypes.c_int, [ctypes.c_int, ctypes.c_int, ctypes.c_int, _D, _D]),
+    ("lbm_bench_steps_per_launch", ctypes.c_int, [ctypes.c_int, ctypes.c_int, ctypes.POINTER(Opts), ctypes.c_int,
+                                                  ctypes.POINTER(ctypes.c_int), ctypes.POINTER(ctypes.c_int)]),
     ("lbm_strerror", ctypes.c_char_p, [ctypes.c_int]),
     ("lbm_last_cuda_error", ctypes.c_char_p, []),
 ]
@@ -361,6 +363,16 @@ def bench_fma_peak(kind: str, device: int = -1, reps: int = 20):
     i = ctypes.c_double()
     _check(lib().lbm_bench_fma_peak(k, device, reps, ctypes.byref(f), ctypes.byref(i)), "lbm_bench_fma_peak")
     return f.value, i.value
+
+
+def bench_steps_per_launch(nx: int, ny: int, sms: int = 0, **opts):
+    """(time steps one launch of step() takes where enough are due, 'step' /
+    'tile' / 'strips'), lbm_bench.h; sms = 0 asks the device."""
+    m, k = ctypes.c_int(), ctypes.c_int()
+    o = default_opts(**opts)
+    _check(lib().lbm_bench_steps_per_launch(nx, ny, ctypes.byref(o), sms, ctypes.byref(m), ctypes.byref(k)),
+           "lbm_bench_steps_per_launch")
+    return m.value, ("step", "tile", "strips")[k.value]
 
 
 def strerror(code: int) -> str:
