@@ -87,17 +87,28 @@ def bytes_per_node(prec, tau_iters=0):
     return BYTES_PER_NODE[prec] - (TAU_BYTES[prec] if tau_iters else 0)
 
 
-def steps_per_launch(prec, layout, tau_iters, staging, N):
-    """Time steps one launch of lbm_step takes on a large N x N cavity: two with
-    FP32 storage in the two-buffer layout from 600,000 nodes on (2,000,000 with
-    the implicit tau), the rule of lbm_strip.cu."""
-    return 2 if prec in ("f32", "f32d") and not layout and not staging and N * N >= (2000000 if tau_iters else 600000) else 1
+def steps_per_launch(prec, layout, tau_iters, staging, N, sms=0):
+    """(time steps one launch of lbm_step takes on an N x N cavity, 'step' /
+    'tile' / 'strips'), as the library has it (lbm_bench_steps_per_launch)."""
+    from paper_2011_15073_gb300 import lbm
+    return lbm.bench_steps_per_launch(N, N, sms=sms, prec=prec, layout=layout, tau_iters=tau_iters, staging=staging)
 
 
-def launch_label(prec, layout, tau_iters, staging, N):
-    if steps_per_launch(prec, layout, tau_iters, staging, N) == 2:
-        return "strip_kernel (two steps per launch)"
-    return step_kernel_name(prec, layout, tau_iters, staging, N)
+def launches_of(k, most):
+    """Launches of k steps where one takes up to `most` (1, 2, 4): from replayed
+    graphs too, whose 64 steps are whole ones."""
+    n = 0
+    for m in (4, 2, 1):
+        if m <= most:
+            n, k = n + k // m, k % m
+    return n
+
+
+def launch_label(prec, layout, tau_iters, staging, N, sms=0):
+    m, kernel = steps_per_launch(prec, layout, tau_iters, staging, N, sms)
+    if kernel == "step":
+        return step_kernel_name(prec, layout, tau_iters, staging, N)
+    return {"strips": "strip_kernel", "tile": "tile_kernel"}[kernel] + f" ({ {2: 'two', 4: 'four'}[m]} steps per launch)"
 CASE = dict(n=0.6, Da=1e-3, Ra=1e5, Pr=6.2, porosity=0.6)
 FALLBACK_HBM_GBS = 6800.0
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "traffic.txt")
@@ -111,7 +122,7 @@ PRECISION_FILE = os.path.join(ROOT, "profiles", "precision_study_512.txt")
 # the files that define the step kernels' arithmetic and which kernel runs
 # (host-only files are left out: they do not change a measured figure)
 RECORD_SOURCES = ("lbm_device.cuh", "lbm_round.cuh", "lbm_step.cuh", "lbm_kernels.cu", "lbm_strip.cuh", "lbm_strip.cu",
-                  "lbm_fixed.cuh", "lbm_collide_fixed.cuh")
+                  "lbm_tile.cu", "lbm_fixed.cuh", "lbm_collide_fixed.cuh")
 
 
 def kernel_source_hash():
@@ -388,8 +399,8 @@ def time_ours(lbm, torch, N, prec, steps, warmup, delta, stream, layout=0, tau_i
         torch.cuda.synchronize()
         total = t0.elapsed_time(t1) / 1e3
         kern = sum(a.elapsed_time(b) for a, b in ev) / 1e3 / (steps * delta)
-        spl = steps_per_launch(prec, layout, tau_iters, staging, N)
-        launches = steps * (delta // spl + delta % spl + 1 + 2)
+        spl = steps_per_launch(prec, layout, tau_iters, staging, N)[0]
+        launches = steps * (launches_of(delta, spl) + 1 + 2)
         return total, kern, launches, nu
     finally:
         cav.close()
@@ -1066,8 +1077,8 @@ def main():
     units = whole_job_units(world, N, delta, args.steps)
     mlups = units / total / 1e6
     peak, peak_src = hbm_peak()
-    # HBM bytes per node update: a launch of two steps reads and writes the state once for both
-    spl = steps_per_launch(prec, args.layout, args.tau_iters, args.staging, N)
+    # HBM bytes per node update: a launch of several steps reads and writes the state once for them
+    spl = steps_per_launch(prec, args.layout, args.tau_iters, args.staging, N)[0]
     bpn_main = bytes_per_node(prec, args.tau_iters) / spl
     achieved = bpn_main * N * N / kern / 1e9
     key_main = prec + (f"@tau{args.tau_iters}" if args.tau_iters else "") + \
@@ -1078,7 +1089,7 @@ def main():
         vs, vd = 2, args.variant_delta
         vp, vl, vt, vg = parse_variant(v)
         tv, kv, _, nuv = time_ours(lbm, torch, N, vp, vs, 1, vd, stream, layout=vl, tau_iters=vt, staging=vg)
-        bpn = bytes_per_node(vp, vt) / steps_per_launch(vp, vl, vt, vg, N)
+        bpn = bytes_per_node(vp, vt) / steps_per_launch(vp, vl, vt, vg, N)[0]
         av = bpn * N * N / kv / 1e9
         variants[v] = {"MLUPS": N * N * vd * vs / tv / 1e6, "kernel_MLUPS": N * N / kv / 1e6,
                        "fused_steps_per_bench_step": vd,
@@ -1098,9 +1109,9 @@ def main():
                                            "peak": peak_inst, "frac": ach / peak_inst,
                                            "fp64_inst_per_node": ipn,
                                            "peak_source": "measured: lbm_bench_fma_peak FP64 FMA throughput"}
-    # launch-bound small grid: one launch per step against replayed step graphs
+    # launch-bound small grid (four steps per launch): launch after launch against replayed step graphs
     small = {"grid": [256, 256], "storage": "f32d", "fused_steps": 2 * 5000}
-    for key, gs in (("MLUPS_one_launch_per_step", -1), ("MLUPS_replayed_graphs", 0)):
+    for key, gs in (("MLUPS_launch_after_launch", -1), ("MLUPS_replayed_graphs", 0)):
         ts, _, _, _ = time_ours(lbm, torch, 256, "f32d", 2, 1, 5000, stream, graph_steps=gs)
         small[key] = 256 * 256 * 5000 * 2 / ts / 1e6
     e2e = None
