@@ -47,12 +47,13 @@ template <int N>
 struct Q {
     int64_t v;
 };
+// Sums modulo 2^64: those of a node that is about to be refused may wrap.
 template <int N>
-__host__ __device__ __forceinline__ Q<N> operator+(Q<N> a, Q<N> b) { return Q<N>{a.v + b.v}; }
+__host__ __device__ __forceinline__ Q<N> operator+(Q<N> a, Q<N> b) { return Q<N>{(int64_t)((uint64_t)a.v + (uint64_t)b.v)}; }
 template <int N>
-__host__ __device__ __forceinline__ Q<N> operator-(Q<N> a, Q<N> b) { return Q<N>{a.v - b.v}; }
+__host__ __device__ __forceinline__ Q<N> operator-(Q<N> a, Q<N> b) { return Q<N>{(int64_t)((uint64_t)a.v - (uint64_t)b.v)}; }
 template <int N>
-__host__ __device__ __forceinline__ Q<N> operator*(int k, Q<N> a) { return Q<N>{k * a.v}; }
+__host__ __device__ __forceinline__ Q<N> operator*(int k, Q<N> a) { return Q<N>{(int64_t)((uint64_t)k * (uint64_t)a.v)}; }
 // a >> k and a << k: the value halved / doubled k times
 template <int N>
 __host__ __device__ __forceinline__ Q<N> operator>>(Q<N> a, int k) { return Q<N>{a.v >> k}; }

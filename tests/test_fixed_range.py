@@ -12,16 +12,21 @@ import pytest
 ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
 
 
-def test_admitted_states_are_right_and_refused_ones_unchanged(tmp_path):
+@pytest.mark.parametrize("flags", [["-O2"], ["-O1", "-Xcompiler", "-fsanitize=signed-integer-overflow,"
+                                             "-fno-sanitize-recover=signed-integer-overflow", "-lubsan"]],
+                         ids=["plain", "overflow-checked"])
+def test_admitted_states_are_right_and_refused_ones_unchanged(tmp_path, flags):
+    """The tests of a node's ranges look at sums that may wrap, which signed
+    integers may not: checked too."""
     nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
     if not os.path.exists(nvcc):
         pytest.skip("nvcc not available")
     exe = str(tmp_path / "fixed_range_check")
     src = os.path.join(ROOT, "tests", "host", "fixed_range_check.cu")
     inc = os.path.join(ROOT, "paper_2011_15073_gb300", "csrc")
-    subprocess.run([nvcc, "-O2", "-std=c++17", "-I", inc, src, "-o", exe], check=True, timeout=300)
+    subprocess.run([nvcc, "-std=c++17", "-I", inc, src, "-o", exe, *flags], check=True, timeout=300)
     r = subprocess.run([exe], capture_output=True, text=True, timeout=300)
-    assert r.returncode == 0 and r.stdout.startswith("OK"), r.stdout[-2000:]
+    assert r.returncode == 0 and r.stdout.startswith("OK"), (r.stdout + r.stderr)[-2000:]
 
 
 # f and g to 1e-12, as every FP64 run against the oracle.  tau: 1e-14 in the
